@@ -39,6 +39,7 @@
 #include "blocks.cuh"
 #include "colour.cuh"
 #include "element.cuh"
+#include "element_fixed.cuh"
 #include "elmat.cuh"
 
 struct nsrhs_mesh {
@@ -86,6 +87,7 @@ struct nsrhs_mesh {
 namespace {
 
 using nsrhs::ElemParams;
+using nsrhs::fixed::FixedParams;
 
 std::mutex g_registry_mutex;
 std::unordered_set<const nsrhs_mesh*> g_registry;
@@ -478,11 +480,22 @@ __device__ __forceinline__ void load_geometry(const R* __restrict__ geom, int64_
 // the per-mesh cache (an 88-byte streamed record), or the node coordinates
 // gathered through the connectivity and formed into the Jacobian in the
 // call itself (Sec. V-B's per-element constant gradients, 43 FP64 operations).
+// get(): into registers; stage(): the cofactors into the scratch slots of the
+// fixed-point routines, 1/detJ and detJ^(-1/3) into registers.
 struct GeomCached {
   const double* __restrict__ geom;
   __device__ __forceinline__ void get(int64_t E, int64_t e, const int32_t v[4], double c[3][3],
                                       double& inv_det, double& rh) const {
     load_geometry(geom, E, e, c, inv_det, rh);
+  }
+  template <int T>
+  __device__ __forceinline__ void stage(const nsrhs::fixed::Scratch<T>& sc, int64_t E, int64_t e,
+                                        const int32_t v[4], double& inv_det, double& rh) const {
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+      nsrhs::cp_async<8>(sc.q + (nsrhs::fixed::kSlotC + q) * T, geom + q * E + e);
+    inv_det = ldg(geom + 9 * E + e);
+    rh = ldg(geom + 10 * E + e);
   }
 };
 struct GeomRecompute {
@@ -497,6 +510,14 @@ struct GeomRecompute {
       for (int d = 0; d < 3; ++d) X[a][d] = __ldg(coords + d * N + v[a]);
     nsrhs::element_geometry<double, double>(X, c, inv_det, rh);
   }
+  template <int T>
+  __device__ __forceinline__ void stage(const nsrhs::fixed::Scratch<T>& sc, int64_t E, int64_t e,
+                                        const int32_t v[4], double& inv_det, double& rh) const {
+    double c[3][3];
+    get(E, e, v, c, inv_det, rh);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) sc.put_real(nsrhs::fixed::kSlotC + q, c[q / 3][q % 3]);
+  }
 };
 
 // A result entry as double: itself, or a float widened with integer
@@ -504,15 +525,14 @@ struct GeomRecompute {
 __device__ __forceinline__ double to_double(double x) { return x; }
 __device__ __forceinline__ double to_double(float x) { return nsrhs::widen_f32(x); }
 
-// FP64 forward of element e: streamed connectivity and cached geometry,
-// gathered nodal (u, p), register-resident element arithmetic, immediate
-// scatter of the 16 entries.
-template <int FLAGS, bool COLOUR, class GS = GeomCached>
-__device__ __forceinline__ void fwd_fp64_element(int64_t N, int64_t E, int64_t e,
-                                                 const int32_t* __restrict__ conn, const GS& gs,
-                                                 const double* __restrict__ up,
-                                                 const ElemParams<double>& P,
-                                                 double* __restrict__ rhs) {
+// FP64 forward of element e on the FP64 pipe: the elements that the block
+// fixed-point routine leaves (element_fixed.cuh). Out of line, so that its
+// registers and code stay out of the common path.
+template <int FLAGS, class GS>
+__device__ __noinline__ void fwd_fp64_plain(int64_t N, int64_t E, int64_t e,
+                                            const int32_t* __restrict__ conn, GS gs,
+                                            const double* __restrict__ up, ElemParams<double> P,
+                                            double* __restrict__ rhs) {
   int32_t v[4];
 #pragma unroll
   for (int a = 0; a < 4; ++a) v[a] = ldg(conn + a * E + e);
@@ -533,43 +553,68 @@ __device__ __forceinline__ void fwd_fp64_element(int64_t N, int64_t E, int64_t e
     for (int k = 0; k < 4; ++k) atomicAdd(rhs + k * N + v[a], F[a][k]);
 }
 
-// FP64 forward, one element per thread over all elements, atomic scatter.
-template <int FLAGS>
-__global__ void __launch_bounds__(kThreads, NSRHS_FWD_MIN_CTAS)
-    fwd_fp64_atomic_kernel(int64_t N, int64_t E, const int32_t* __restrict__ conn,
-                           const double* __restrict__ geom, const double* __restrict__ up,
-                           ElemParams<double> P, double* __restrict__ rhs) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < E;
-       e += (int64_t)gridDim.x * blockDim.x)
-    fwd_fp64_element<FLAGS, false>(N, E, e, conn, GeomCached{geom}, up, P, rhs);
-}
+// Adds component k of an element's entries to the nodal rows.
+struct AddEntries {
+  double* __restrict__ out;
+  int64_t N;
+  const int32_t* v;
+  __device__ __forceinline__ void operator()(int k, const double f[4]) const {
+#pragma unroll
+    for (int a = 0; a < 4; ++a) atomicAdd(out + k * N + v[a], f[a]);
+  }
+};
 
-// FP64 forward with the element geometry formed from the gathered node
-// coordinates in the call (no cached geometry read), atomic scatter.
-template <int FLAGS>
-__global__ void __launch_bounds__(kThreads, NSRHS_FWD_MIN_CTAS)
-    fwd_fp64_recompute_kernel(int64_t N, int64_t E, const int32_t* __restrict__ conn,
-                              const double* __restrict__ coords, const double* __restrict__ up,
-                              ElemParams<double> P, double* __restrict__ rhs) {
-  const GeomRecompute gs{coords, N};
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < E;
-       e += (int64_t)gridDim.x * blockDim.x)
-    fwd_fp64_element<FLAGS, false>(N, E, e, conn, gs, up, P, rhs);
-}
+// The double-precision kernels run one warp per CTA: their scratch in shared
+// memory (14 KB a warp) and 128 registers let 15 warps share an SM, and a
+// small mesh spreads over as many SMs as it has warps. 64 and 128 threads
+// per CTA measured the same on large meshes (128^3: 2.79, 2.79, 2.91 ms).
+constexpr int kFixedThreads = 32;
 
-// FP64 forward over the elements [e0, e1) of one colour of the colour-major
-// copy (row stride E). No two elements of a colour share a node, so every
-// address receives at most one atomic in the launch, and the colour order
-// fixes the summation order: the result is bitwise reproducible.
-template <int FLAGS>
-__global__ void __launch_bounds__(kThreads, NSRHS_FWD_COLOUR_MIN_CTAS)
-    fwd_fp64_colour_kernel(int64_t N, int64_t E, int64_t e0, int64_t e1,
-                           const int32_t* __restrict__ conn, const double* __restrict__ geom,
-                           const double* __restrict__ up, ElemParams<double> P,
-                           double* __restrict__ rhs) {
-  for (int64_t e = e0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < e1;
-       e += (int64_t)gridDim.x * blockDim.x)
-    fwd_fp64_element<FLAGS, true>(N, E, e, conn, GeomCached{geom}, up, P, rhs);
+// FP64 forward of the elements [e0, e1) (row stride E), one per thread:
+// streamed connectivity, geometry from GS, gathered nodal (u, p), block
+// fixed-point arithmetic (element_fixed.cuh), immediate scatter of the 16
+// entries with atomics. Two uses: all elements of the mesh; or one colour of
+// the colour-major copy, where no two elements share a node, so that every
+// address receives at most one atomic in the launch and the colour order
+// fixes the summation order (bitwise reproducible).
+//
+// Bound by instruction issue (ALU pipe 60 % busy, 4650 instructions a warp at
+// 0.53 per clock and sub-partition), where the FP64 form kept the FP64 pipe
+// 90 % busy with 344 FP64 instructions (64 clocks of a sub-partition each):
+// 256^3 61.4 -> 22.7 ms.
+//
+// plain: every element on the FP64 pipe (parameters outside the fixed-point
+// range).
+template <int FLAGS, class GS>
+__global__ void __launch_bounds__(kFixedThreads, 15)
+    fwd_fp64_kernel(int64_t N, int64_t E, int64_t e0, int64_t e1,
+                    const int32_t* __restrict__ conn, GS gs, const double* __restrict__ up,
+                    const __grid_constant__ FixedParams P, bool plain,
+                    double* __restrict__ rhs) {
+  namespace fx = nsrhs::fixed;
+  constexpr int T = kFixedThreads;
+  constexpr int slots = (FLAGS & nsrhs::kSkew) ? fx::kFwdSlotsSkew : fx::kFwdSlots;
+  __shared__ int64_t sq[slots * T];
+  __shared__ int32_t sw[fx::kFwdWords * T];
+  const fx::Scratch<T> sc{sq + threadIdx.x, sw + threadIdx.x};
+  for (int64_t e = e0 + blockIdx.x * (int64_t)T + threadIdx.x; e < e1; e += (int64_t)gridDim.x * T) {
+    if (!plain) {
+      int32_t v[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) v[a] = ldg(conn + a * E + e);
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          nsrhs::cp_async<8>(sc.q + (fx::kSlotU + 4 * i + a) * T, up + i * N + v[a]);
+      double inv_det, rh;
+      gs.stage(sc, E, e, v, inv_det, rh);
+      nsrhs::cp_async_commit();
+      nsrhs::cp_async_wait<0>();
+      if (fx::element_rhs_fixed<FLAGS, T>(sc, inv_det, rh, P, AddEntries{rhs, N, v})) continue;
+    }
+    fwd_fp64_plain<FLAGS, GS>(N, E, e, conn, gs, up, P.P, rhs);
+  }
 }
 
 // Element-matrix comparison kernel: the same RHS through a full 16x16
@@ -913,6 +958,20 @@ bool block_smem_fits(const nsrhs_mesh* m, const nsrhs_params* p, int W, int entr
 bool recompute_supported(const nsrhs_params* p) {
   return p->precision == NSRHS_FP64 &&
          (p->scatter == NSRHS_SCATTER_AUTO || p->scatter == NSRHS_SCATTER_ATOMIC);
+}
+
+template <class R>
+ElemParams<R> elem_params(const nsrhs_params* p);
+
+FixedParams fixed_params(const nsrhs_params* p) {
+  return nsrhs::fixed::make_fixed_params(elem_params<double>(p), p->convection == NSRHS_SKEW);
+}
+
+// Grid of a one-warp-per-CTA kernel over n elements: several waves of the 15
+// resident CTAs per SM.
+unsigned fixed_grid(int64_t n, int device) {
+  const int64_t need = (n + kFixedThreads - 1) / kFixedThreads;
+  return (unsigned)std::max<int64_t>(1, std::min(need, (int64_t)sm_count(device) * 64));
 }
 
 template <class R>
@@ -1375,11 +1434,12 @@ nsrhs_status nsrhs_assemble(const nsrhs_mesh* m, const nsrhs_params* p, const vo
     return NSRHS_EUNSUPPORTED;
   NSRHS_TRY(cudaMemsetAsync(rhs, 0, sizeof(double) * 4 * N, s));
   if (p->geometry == NSRHS_GEOM_RECOMPUTE) {
-    auto P = elem_params<double>(p);
+    const FixedParams P = fixed_params(p);
     with_flags(flags, [&](auto fl) {
-      fwd_fp64_recompute_kernel<decltype(fl)::value><<<grid_for(E, m->device, 16), kThreads, 0,
-                                                       s>>>(N, E, m->conn, m->coords,
-                                                            (const double*)up, P, rhs);
+      fwd_fp64_kernel<decltype(fl)::value, GeomRecompute>
+          <<<fixed_grid(E, m->device), kFixedThreads, 0, s>>>(
+              N, E, 0, E, m->conn, GeomRecompute{m->coords, N}, (const double*)up, P,
+              !P.in_range, rhs);
     });
     return cuda_status(cudaGetLastError());
   }
@@ -1424,10 +1484,12 @@ nsrhs_status nsrhs_assemble(const nsrhs_mesh* m, const nsrhs_params* p, const vo
       const int64_t e0 = m->col_off[k], e1 = m->col_off[k + 1];
       const unsigned grid = grid_for(e1 - e0, m->device, 16);
       if (p->precision == NSRHS_FP64) {
-        auto P = elem_params<double>(p);
+        const FixedParams P = fixed_params(p);
         with_flags(flags, [&](auto fl) {
-          fwd_fp64_colour_kernel<decltype(fl)::value><<<grid, kThreads, 0, s>>>(
-              N, E, e0, e1, m->col_conn, m->col_geom, (const double*)up, P, rhs);
+          fwd_fp64_kernel<decltype(fl)::value, GeomCached>
+              <<<fixed_grid(e1 - e0, m->device), kFixedThreads, 0, s>>>(
+                  N, E, e0, e1, m->col_conn, GeomCached{m->col_geom}, (const double*)up, P,
+                  !P.in_range, rhs);
         });
       } else {
         auto P = elem_params<float>(p);
@@ -1480,10 +1542,12 @@ nsrhs_status nsrhs_assemble(const nsrhs_mesh* m, const nsrhs_params* p, const vo
   }
   const unsigned grid = grid_for(E, m->device, 16);
   if (p->precision == NSRHS_FP64) {
-    auto P = elem_params<double>(p);
+    const FixedParams P = fixed_params(p);
     with_flags(flags, [&](auto fl) {
-      fwd_fp64_atomic_kernel<decltype(fl)::value>
-          <<<grid, kThreads, 0, s>>>(N, E, m->conn, m->geom, (const double*)up, P, rhs);
+      fwd_fp64_kernel<decltype(fl)::value, GeomCached>
+          <<<fixed_grid(E, m->device), kFixedThreads, 0, s>>>(
+              N, E, 0, E, m->conn, GeomCached{m->geom}, (const double*)up, P,
+              !P.in_range, rhs);
     });
   } else {
     auto P = elem_params<float>(p);
