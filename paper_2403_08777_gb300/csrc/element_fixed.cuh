@@ -56,6 +56,8 @@ struct FixedParams {
 
 constexpr int64_t kBeta62 = 0x13c6ef372fe94f83ll;       // beta 2^62
 constexpr int64_t kBeta61 = 0x9e3779b97f4a7c2ll;        // beta 2^61
+constexpr int64_t kQB61 = 0x46c1b47480244d9ll;          // QB 2^61
+constexpr int64_t kEightFifteenths60 = 0x888888888888889ll;  // (8/15) 2^60
 constexpr int64_t kTwoThirds61 = 0x1555555555555555ll;  // (2/3) 2^61; 1/24 = 2^-4 2/3
 
 // Per-thread scratch in shared memory: 64-bit slots and 32-bit words, the
@@ -108,6 +110,11 @@ __device__ __forceinline__ int64_t beta_sum_wide(int64_t V) {
   return mulx<3>(limb(kBeta61), limb(V >> 2)) * 4;
 }
 
+// QB V, likewise.
+__device__ __forceinline__ int64_t qb_sum(int64_t V) {
+  return mulx<3>(limb(kQB61), limb(V >> 2)) * 4;
+}
+
 // |v|^2 of the vector v_i 2^(eu_i - 59), |v_i| < 2^60.2, as a double;
 // eum = max eu_i. The vector is normalised first: a Gauss point may be nearly
 // at rest.
@@ -153,12 +160,14 @@ __device__ __forceinline__ void gauss_matrices(const Acc q[6], int64_t T[3], int
 // The row base + sum_j K_j C_a,j with base = +-tr R / 24 (third = +-(2/3) 2^60)
 // and K_j = sum_k sT_k R_jk + sg r_j, from the rows R at slot sR (exponents
 // eR_j + t_k) and the vector r at slot sr (exponents t_j and, with sg's, er).
-// Returns the exponent for to_double.
+// sE, sT0: the words of eR and t; sk: three free slots. Returns the exponent
+// for to_double.
 template <int THREADS>
-__device__ __forceinline__ int trace_row(const Scratch<THREADS>& sc, int sR, int sr,
+__device__ __forceinline__ int trace_row(const Scratch<THREADS>& sc, int sR, int sr, int sE, int sT0,
                                          const int eR[3], const int t[3], int tmax,
                                          const Limb sT[3], int eT, const Limb& sg, int er,
-                                         int64_t third, Limb K[3], int64_t& base) {
+                                         int64_t third, int sk, Limb K[3],
+                                         int64_t& base) {
   // tr R, often much smaller than its terms: summed unshifted (below 2^62.6)
   // and normalised
   const int et = imax(eR[0] + t[0], imax(eR[1] + t[1], eR[2] + t[2]));
@@ -173,21 +182,25 @@ __device__ __forceinline__ int trace_row(const Scratch<THREADS>& sc, int sR, int
   int e = imax(ec, er + 2 * tmax);
 #pragma unroll
   for (int j = 0; j < 3; ++j) e = imax(e, eR[j] + t[j] + eT);
-  int64_t k[3];
-#pragma unroll
+  uint32_t m = 0;
+#pragma unroll 1
   for (int j = 0; j < 3; ++j) {
     Limb g[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) g[i] = limb(sc.get(sR + 3 * j + i));
-    k[j] = shr(dot3x<2>(sT[0], g[0], sT[1], g[1], sT[2], g[2]), e - (eR[j] + eT + t[j])) +
-           shr(mulx<2>(sg, limb(sc.get(sr + j))), e - (er + 2 * t[j]));
+    const int tj = sc.word(sT0 + j);
+    const int64_t k =
+        shr(dot3x<2>(sT[0], g[0], sT[1], g[1], sT[2], g[2]), e - (sc.word(sE + j) + eT + tj)) +
+        shr(mulx<2>(sg, limb(sc.get(sr + j))), e - (er + 2 * tj));
+    m |= mag(k);
+    sc.put(sk + j, k);
   }
   base = shr_round(c0, e - ec);  // the K_j may cancel in sum_j K_j C_a,j
   // |k| < 2^61, |base| < 2^60
-  const int n = norm_shift(mag(k[0]) | mag(k[1]) | mag(k[2]) | mag(base));
+  const int n = norm_shift(m | mag(base));
   base = shl(base, n);
 #pragma unroll
-  for (int j = 0; j < 3; ++j) K[j] = limb(shl(k[j], n));
+  for (int j = 0; j < 3; ++j) K[j] = limb(shl(sc.get(sk + j), n));
   return e - n + 4;
 }
 
@@ -493,8 +506,8 @@ __device__ __forceinline__ bool element_rhs_fixed(const Scratch<THREADS>& sc, do
       int es;
       const int64_t sm = scalar_fixed(stau, es);
       const Limb sg = limb(mul8(limb(mul8(inv, nsrhs::fixed::limb(-kTwoThirds61))), limb(sm * 2)));
-      e = trace_row(sc, kSlotG, kSlotG + 9, eG, t, tmax, sT, eT, sg, einv - 4 + es + egp,
-                    -kTwoThirds61 / 2, Kl, base);
+      e = trace_row(sc, kSlotG, kSlotG + 9, kWordEg, kWordT, eG, t, tmax, sT, eT, sg,
+                    einv - 4 + es + egp, -kTwoThirds61 / 2, kSlotX, Kl, base);
     }
     int64_t y[4];
     y[0] = base;

@@ -40,6 +40,7 @@
 #include "colour.cuh"
 #include "element.cuh"
 #include "element_fixed.cuh"
+#include "element_fixed_vjp.cuh"
 #include "elmat.cuh"
 
 struct nsrhs_mesh {
@@ -101,23 +102,6 @@ constexpr int kThreads = 128;
 constexpr int kGeomRows = 11;
 // Block-kernel grids: at most a full SM's worth of threads (2048) per SM.
 constexpr int kBlockCtasPerSm = 2048 / nsrhs::kBlockElems > 0 ? 2048 / nsrhs::kBlockElems : 1;
-
-// Minimum resident CTAs per SM requested from the compiler (register cap) for
-// the FP64 element kernels; measured choices, overridable at build time.
-#ifndef NSRHS_FWD_MIN_CTAS
-#define NSRHS_FWD_MIN_CTAS 1
-#endif
-#ifndef NSRHS_VJP_MIN_CTAS
-#define NSRHS_VJP_MIN_CTAS 1
-#endif
-// The coloured FP64 kernels: capped so that as many CTAs fit per SM as for
-// the atomic kernels.
-#ifndef NSRHS_FWD_COLOUR_MIN_CTAS
-#define NSRHS_FWD_COLOUR_MIN_CTAS 3
-#endif
-#ifndef NSRHS_VJP_COLOUR_MIN_CTAS
-#define NSRHS_VJP_COLOUR_MIN_CTAS 2
-#endif
 
 int sm_count(int device) {
   int n = 0;
@@ -491,9 +475,9 @@ struct GeomCached {
   template <int T>
   __device__ __forceinline__ void stage(const nsrhs::fixed::Scratch<T>& sc, int64_t E, int64_t e,
                                         const int32_t v[4], double& inv_det, double& rh) const {
+    static_assert(nsrhs::fixed::kSlotC == 0 && nsrhs::fixed::kVjpC == 0, "cofactor slots");
 #pragma unroll
-    for (int q = 0; q < 9; ++q)
-      nsrhs::cp_async<8>(sc.q + (nsrhs::fixed::kSlotC + q) * T, geom + q * E + e);
+    for (int q = 0; q < 9; ++q) nsrhs::cp_async<8>(sc.q + q * T, geom + q * E + e);
     inv_det = ldg(geom + 9 * E + e);
     rh = ldg(geom + 10 * E + e);
   }
@@ -516,14 +500,9 @@ struct GeomRecompute {
     double c[3][3];
     get(E, e, v, c, inv_det, rh);
 #pragma unroll
-    for (int q = 0; q < 9; ++q) sc.put_real(nsrhs::fixed::kSlotC + q, c[q / 3][q % 3]);
+    for (int q = 0; q < 9; ++q) sc.put_real(q, c[q / 3][q % 3]);
   }
 };
-
-// A result entry as double: itself, or a float widened with integer
-// operations (no FP64 instruction).
-__device__ __forceinline__ double to_double(double x) { return x; }
-__device__ __forceinline__ double to_double(float x) { return nsrhs::widen_f32(x); }
 
 // FP64 forward of element e on the FP64 pipe: the elements that the block
 // fixed-point routine leaves (element_fixed.cuh). Out of line, so that its
@@ -553,7 +532,13 @@ __device__ __noinline__ void fwd_fp64_plain(int64_t N, int64_t E, int64_t e,
     for (int k = 0; k < 4; ++k) atomicAdd(rhs + k * N + v[a], F[a][k]);
 }
 
-// Adds component k of an element's entries to the nodal rows.
+// v[a] for a run-time a, from registers.
+__device__ __forceinline__ int32_t pick(const int32_t v[4], int a) {
+  return a < 2 ? (a == 0 ? v[0] : v[1]) : (a == 2 ? v[2] : v[3]);
+}
+
+// Adds component k of an element's entries to the nodal rows: all four nodes',
+// or that of node a.
 struct AddEntries {
   double* __restrict__ out;
   int64_t N;
@@ -561,6 +546,9 @@ struct AddEntries {
   __device__ __forceinline__ void operator()(int k, const double f[4]) const {
 #pragma unroll
     for (int a = 0; a < 4; ++a) atomicAdd(out + k * N + v[a], f[a]);
+  }
+  __device__ __forceinline__ void operator()(int k, int a, double f) const {
+    atomicAdd(out + k * N + pick(v, a), f);
   }
 };
 
@@ -581,7 +569,7 @@ constexpr int kFixedThreads = 32;
 // Bound by instruction issue (ALU pipe 60 % busy, 4650 instructions a warp at
 // 0.53 per clock and sub-partition), where the FP64 form kept the FP64 pipe
 // 90 % busy with 344 FP64 instructions (64 clocks of a sub-partition each):
-// 256^3 61.4 -> 22.7 ms.
+// 256^3 61.3 -> 22.7 ms.
 //
 // plain: every element on the FP64 pipe (parameters outside the fixed-point
 // range).
@@ -700,16 +688,16 @@ __global__ void __launch_bounds__(kThreads)
     fwd_mixed_element<FLAGS, true>(N, E, e, conn, rec, up, P, rhs);
 }
 
-// FP64 vector-Jacobian product of element e: gather the cotangent at the
-// element's nodes (the reverse of the scatter), recompute the element, run
-// the reverse sweep, scatter-add the gradient (the reverse of the gather).
-template <int FLAGS, bool COLOUR, class GS = GeomCached>
-__device__ __forceinline__ void vjp_fp64_element(int64_t N, int64_t E, int64_t e,
-                                                 const int32_t* __restrict__ conn, const GS& gs,
-                                                 const double* __restrict__ up,
-                                                 const double* __restrict__ cot,
-                                                 const ElemParams<double>& P,
-                                                 double* __restrict__ grad) {
+// FP64 vector-Jacobian product of element e on the FP64 pipe (the elements
+// that the fixed-point routine leaves): gather the cotangent at the element's
+// nodes (the reverse of the scatter), recompute the element, run the reverse
+// sweep, scatter-add the gradient (the reverse of the gather).
+template <int FLAGS, class GS>
+__device__ __noinline__ void vjp_fp64_plain(int64_t N, int64_t E, int64_t e,
+                                            const int32_t* __restrict__ conn, GS gs,
+                                            const double* __restrict__ up,
+                                            const double* __restrict__ cot, ElemParams<double> P,
+                                            double* __restrict__ grad) {
   int32_t v[4];
 #pragma unroll
   for (int a = 0; a < 4; ++a) v[a] = ldg(conn + a * E + e);
@@ -734,40 +722,56 @@ __device__ __forceinline__ void vjp_fp64_element(int64_t N, int64_t E, int64_t e
   }
 }
 
-template <int FLAGS>
-__global__ void __launch_bounds__(kThreads, NSRHS_VJP_MIN_CTAS)
-    vjp_fp64_atomic_kernel(int64_t N, int64_t E, const int32_t* __restrict__ conn,
-                           const double* __restrict__ geom, const double* __restrict__ up,
-                           const double* __restrict__ cot, ElemParams<double> P,
-                           double* __restrict__ grad) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < E;
-       e += (int64_t)gridDim.x * blockDim.x)
-    vjp_fp64_element<FLAGS, false>(N, E, e, conn, GeomCached{geom}, up, cot, P, grad);
-}
+// An element's nodal velocities in global memory, for the parts of the
+// fixed-point adjoint that take them as doubles.
+struct NodalVelocity {
+  const double* __restrict__ up;
+  int64_t N;
+  const int32_t* v;
+  __device__ __forceinline__ double operator()(int i, int a) const {
+    return ldg(up + i * N + pick(v, a));
+  }
+};
 
-// FP64 adjoint with the element geometry formed from the gathered node
-// coordinates in the call, atomic scatter.
-template <int FLAGS>
-__global__ void __launch_bounds__(kThreads, NSRHS_VJP_MIN_CTAS)
-    vjp_fp64_recompute_kernel(int64_t N, int64_t E, const int32_t* __restrict__ conn,
-                              const double* __restrict__ coords, const double* __restrict__ up,
-                              const double* __restrict__ cot, ElemParams<double> P,
-                              double* __restrict__ grad) {
-  const GeomRecompute gs{coords, N};
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < E;
-       e += (int64_t)gridDim.x * blockDim.x)
-    vjp_fp64_element<FLAGS, false>(N, E, e, conn, gs, up, cot, P, grad);
-}
-
-template <int FLAGS>
-__global__ void __launch_bounds__(kThreads, NSRHS_VJP_COLOUR_MIN_CTAS)
-    vjp_fp64_colour_kernel(int64_t N, int64_t E, int64_t e0, int64_t e1,
-                           const int32_t* __restrict__ conn, const double* __restrict__ geom,
-                           const double* __restrict__ up, const double* __restrict__ cot,
-                           ElemParams<double> P, double* __restrict__ grad) {
-  for (int64_t e = e0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < e1;
-       e += (int64_t)gridDim.x * blockDim.x)
-    vjp_fp64_element<FLAGS, true>(N, E, e, conn, GeomCached{geom}, up, cot, P, grad);
+// FP64 adjoint of the elements [e0, e1) (row stride E), one per thread; the
+// two uses, GS and plain as in fwd_fp64_kernel. Integer and FP64 pipe share
+// the sweep (element_fixed_vjp.cuh): FP64 pipe 60 % busy, ALU 37 %, 0.38
+// instructions per clock and sub-partition with the 10 warps per SM that
+// 22 KB of scratch a warp allow, where the FP64 form kept the FP64 pipe 90 %
+// busy with 648 instructions: 256^3 114.4 -> 60.5 ms.
+template <int FLAGS, class GS>
+__global__ void __launch_bounds__(kFixedThreads, 10)
+    vjp_fp64_kernel(int64_t N, int64_t E, int64_t e0, int64_t e1,
+                    const int32_t* __restrict__ conn, GS gs, const double* __restrict__ up,
+                    const double* __restrict__ cot, const __grid_constant__ FixedParams P,
+                    bool plain, double* __restrict__ grad) {
+  namespace fx = nsrhs::fixed;
+  constexpr int T = kFixedThreads;
+  __shared__ int64_t sq[fx::kVjpSlots * T];
+  __shared__ int32_t sw[fx::kVjpWords * T];
+  const fx::Scratch<T> sc{sq + threadIdx.x, sw + threadIdx.x};
+  for (int64_t e = e0 + blockIdx.x * (int64_t)T + threadIdx.x; e < e1; e += (int64_t)gridDim.x * T) {
+    if (!plain) {
+      int32_t v[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) v[a] = ldg(conn + a * E + e);
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          nsrhs::cp_async<8>(sc.q + (fx::kVjpU + 4 * i + a) * T, up + i * N + v[a]);
+          nsrhs::cp_async<8>(sc.q + (fx::kVjpW + 4 * i + a) * T, cot + i * N + v[a]);
+        }
+      double inv_det, rh;
+      gs.stage(sc, E, e, v, inv_det, rh);
+      nsrhs::cp_async_commit();
+      nsrhs::cp_async_wait<0>();
+      if (fx::element_vjp_fixed<FLAGS, T>(sc, inv_det, rh, P, NodalVelocity{up, N, v},
+                                          AddEntries{grad, N, v}))
+        continue;
+    }
+    vjp_fp64_plain<FLAGS, GS>(N, E, e, conn, gs, up, cot, P.P, grad);
+  }
 }
 
 // Mixed-precision vector-Jacobian product of element e: float (u, p), float
@@ -829,22 +833,25 @@ __global__ void __launch_bounds__(kThreads)
     vjp_mixed_element<FLAGS, true>(N, E, e, conn, rec, up, cot, P, grad);
 }
 
-// The RHS and the vector-Jacobian product at the same state in one pass
+// The mixed RHS and vector-Jacobian product at the same state in one pass
 // (element_rhs_vjp): one gather of (u, p) and the cotangent, one geometry
-// read, the forward intermediates computed once; R = double (FP64) or float
-// (mixed: float arithmetic, double accumulation by integer widening).
-template <class R, int FLAGS, class G>
-__global__ void __launch_bounds__(kThreads, NSRHS_VJP_MIN_CTAS)
-    rhs_vjp_atomic_kernel(int64_t N, int64_t E, const int32_t* __restrict__ conn,
-                          const G* __restrict__ geom, const R* __restrict__ up,
-                          const R* __restrict__ cot, ElemParams<R> P, double* __restrict__ rhs,
-                          double* __restrict__ grad) {
+// read, the forward intermediates computed once; float arithmetic, double
+// accumulation by integer widening. (The FP64 form runs its forward and its
+// adjoint kernel one after the other: fixed-point forward and adjoint, 23 + 60
+// ms at 256^3, against 141 ms for one FP64 pass.)
+template <int FLAGS>
+__global__ void __launch_bounds__(kThreads)
+    rhs_vjp_mixed_atomic_kernel(int64_t N, int64_t E, const int32_t* __restrict__ conn,
+                                const nsrhs::RecChunk* __restrict__ rec,
+                                const float* __restrict__ up, const float* __restrict__ cot,
+                                ElemParams<float> P, double* __restrict__ rhs,
+                                double* __restrict__ grad) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < E;
        e += (int64_t)gridDim.x * blockDim.x) {
     int32_t v[4];
 #pragma unroll
     for (int a = 0; a < 4; ++a) v[a] = ldg(conn + a * E + e);
-    R u[4][3], p[4], w[4][4];
+    float u[4][3], p[4], w[4][4];
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
 #pragma unroll
@@ -853,18 +860,17 @@ __global__ void __launch_bounds__(kThreads, NSRHS_VJP_MIN_CTAS)
 #pragma unroll
       for (int k = 0; k < 4; ++k) w[a][k] = ldg(cot + k * N + v[a]);
     }
-    R c[3][3], inv_det, rh;
-    nsrhs::block_geometry(reinterpret_cast<const nsrhs::RecChunk*>(geom),
-                          reinterpret_cast<const double*>(geom), E, e, c, inv_det, rh);
-    R F[4][4], gu[4][3], gp[4];
-    nsrhs::element_rhs_vjp<R, FLAGS>(c, inv_det, rh, u, p, w, P, F, gu, gp);
+    float c[3][3], inv_det, rh;
+    nsrhs::load_rec_geometry(rec, e, c, inv_det, rh);
+    float F[4][4], gu[4][3], gp[4];
+    nsrhs::element_rhs_vjp<float, FLAGS>(c, inv_det, rh, u, p, w, P, F, gu, gp);
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) atomicAdd(rhs + k * N + v[a], to_double(F[a][k]));
+      for (int k = 0; k < 4; ++k) atomicAdd(rhs + k * N + v[a], nsrhs::widen_f32(F[a][k]));
 #pragma unroll
-      for (int i = 0; i < 3; ++i) atomicAdd(grad + i * N + v[a], to_double(gu[a][i]));
-      atomicAdd(grad + 3 * N + v[a], to_double(gp[a]));
+      for (int i = 0; i < 3; ++i) atomicAdd(grad + i * N + v[a], nsrhs::widen_f32(gu[a][i]));
+      atomicAdd(grad + 3 * N + v[a], nsrhs::widen_f32(gp[a]));
     }
   }
 }
@@ -1580,12 +1586,12 @@ nsrhs_status nsrhs_assemble_vjp(const nsrhs_mesh* m, const nsrhs_params* p, cons
   NSRHS_TRY(cudaMemsetAsync(grad, 0, sizeof(double) * 4 * N, s));
   const int flags = formulation_flags(p);
   if (p->geometry == NSRHS_GEOM_RECOMPUTE) {
-    auto P = elem_params<double>(p);
+    const FixedParams P = fixed_params(p);
     with_flags(flags, [&](auto fl) {
-      vjp_fp64_recompute_kernel<decltype(fl)::value><<<grid_for(E, m->device, 16), kThreads, 0,
-                                                       s>>>(N, E, m->conn, m->coords,
-                                                            (const double*)up,
-                                                            (const double*)cot, P, grad);
+      vjp_fp64_kernel<decltype(fl)::value, GeomRecompute>
+          <<<fixed_grid(E, m->device), kFixedThreads, 0, s>>>(
+              N, E, 0, E, m->conn, GeomRecompute{m->coords, N}, (const double*)up,
+              (const double*)cot, P, !P.in_range, grad);
     });
     return cuda_status(cudaGetLastError());
   }
@@ -1645,11 +1651,12 @@ nsrhs_status nsrhs_assemble_vjp(const nsrhs_mesh* m, const nsrhs_params* p, cons
       const int64_t e0 = m->col_off[k], e1 = m->col_off[k + 1];
       const unsigned grid = grid_for(e1 - e0, m->device, 16);
       if (p->precision == NSRHS_FP64) {
-        auto P = elem_params<double>(p);
+        const FixedParams P = fixed_params(p);
         with_flags(formulation_flags(p), [&](auto fl) {
-          vjp_fp64_colour_kernel<decltype(fl)::value><<<grid, kThreads, 0, s>>>(
-              N, E, e0, e1, m->col_conn, m->col_geom, (const double*)up, (const double*)cot, P,
-              grad);
+          vjp_fp64_kernel<decltype(fl)::value, GeomCached>
+              <<<fixed_grid(e1 - e0, m->device), kFixedThreads, 0, s>>>(
+                  N, E, e0, e1, m->col_conn, GeomCached{m->col_geom}, (const double*)up,
+                  (const double*)cot, P, !P.in_range, grad);
         });
       } else {
         auto P = elem_params<float>(p);
@@ -1665,10 +1672,12 @@ nsrhs_status nsrhs_assemble_vjp(const nsrhs_mesh* m, const nsrhs_params* p, cons
   }
   const unsigned grid = grid_for(E, m->device, 16);
   if (p->precision == NSRHS_FP64) {
-    auto P = elem_params<double>(p);
+    const FixedParams P = fixed_params(p);
     with_flags(formulation_flags(p), [&](auto fl) {
-      vjp_fp64_atomic_kernel<decltype(fl)::value><<<grid, kThreads, 0, s>>>(
-          N, E, m->conn, m->geom, (const double*)up, (const double*)cot, P, grad);
+      vjp_fp64_kernel<decltype(fl)::value, GeomCached>
+          <<<fixed_grid(E, m->device), kFixedThreads, 0, s>>>(
+              N, E, 0, E, m->conn, GeomCached{m->geom}, (const double*)up, (const double*)cot, P,
+              !P.in_range, grad);
     });
   } else {
     auto P = elem_params<float>(p);
@@ -1748,18 +1757,23 @@ nsrhs_status nsrhs_assemble_rhs_vjp(const nsrhs_mesh* m, const nsrhs_params* p, 
     }
     return cuda_status(err);
   }
-  const unsigned grid = grid_for(E, m->device, 16);
   if (p->precision == NSRHS_FP64) {
-    auto P = elem_params<double>(p);
+    // the forward and the adjoint kernel, one after the other
+    const FixedParams P = fixed_params(p);
     with_flags(flags, [&](auto fl) {
-      rhs_vjp_atomic_kernel<double, decltype(fl)::value, double><<<grid, kThreads, 0, s>>>(
-          N, E, m->conn, m->geom, (const double*)up, (const double*)cot, P, rhs, grad);
+      constexpr int F = decltype(fl)::value;
+      const unsigned fgrid = fixed_grid(E, m->device);
+      fwd_fp64_kernel<F, GeomCached><<<fgrid, kFixedThreads, 0, s>>>(
+          N, E, 0, E, m->conn, GeomCached{m->geom}, (const double*)up, P, !P.in_range, rhs);
+      vjp_fp64_kernel<F, GeomCached><<<fgrid, kFixedThreads, 0, s>>>(
+          N, E, 0, E, m->conn, GeomCached{m->geom}, (const double*)up, (const double*)cot, P,
+          !P.in_range, grad);
     });
   } else {
     auto P = elem_params<float>(p);
     with_flags(flags, [&](auto fl) {
-      rhs_vjp_atomic_kernel<float, decltype(fl)::value, nsrhs::RecChunk>
-          <<<grid, kThreads, 0, s>>>(N, E, m->conn, m->rec, (const float*)up, (const float*)cot, P, rhs, grad);
+      rhs_vjp_mixed_atomic_kernel<decltype(fl)::value><<<grid_for(E, m->device, 16), kThreads, 0, s>>>(
+          N, E, m->conn, m->rec, (const float*)up, (const float*)cot, P, rhs, grad);
     });
   }
   return cuda_status(cudaGetLastError());

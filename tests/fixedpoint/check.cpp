@@ -14,12 +14,13 @@
 #include <random>
 
 #include "../../paper_2403_08777_gb300/csrc/element_fixed.cuh"
+#include "../../paper_2403_08777_gb300/csrc/element_fixed_vjp.cuh"
 
 using namespace nsrhs;
 using fixed::limb;
 
 // The element's right-hand side at the Gauss points, term by term, in long
-// double.
+// double (or complex long double, for derivatives by the complex step).
 typedef long double ld;
 static ld real(ld x) { return x; }
 static ld real(const std::complex<ld>& x) { return x.real(); }
@@ -201,6 +202,7 @@ struct Keep {
   void operator()(int k, const double f[4]) const {
     for (int a = 0; a < 4; ++a) F[a][k] = f[a];
   }
+  void operator()(int k, int a, double f) const { F[a][k] = f; }
 };
 static void stage(const Element& q, int64_t* slots) {
   for (int k = 0; k < 9; ++k) std::memcpy(slots + fixed::kSlotC + k, &q.c[k / 3][k % 3], 8);
@@ -242,11 +244,58 @@ static void routine(int kind, int n) {
       say(k < 3 ? "momentum" : "continuity", FLAGS, kind, std::sqrt(e[k] / norm[k]),
           1.1 * std::sqrt(d[k] / norm[k]));
 }
+// The reverse sweep against complex-step derivatives of the reference.
+template <int FLAGS>
+static void adjoint(int kind, int n) {
+  typedef std::complex<ld> cld;
+  double e[4] = {}, d[4] = {}, norm[4] = {};
+  int left = 0;
+  for (int it = 0; it < n; ++it) {
+    const Element q = make(kind, it);
+    const auto FP = fixed::make_fixed_params(q.P, (FLAGS & kSkew) != 0);
+    double gu[4][3], gp[4], G[4][4];
+    element_vjp<double, FLAGS>(q.c, q.inv, q.rh, q.u, q.p, q.w, q.P, gu, gp);
+    int64_t slots[128];
+    int32_t words[32];
+    for (int k = 0; k < 9; ++k) std::memcpy(slots + fixed::kVjpC + k, &q.c[k / 3][k % 3], 8);
+    for (int a = 0; a < 4; ++a) {
+      for (int i = 0; i < 3; ++i) std::memcpy(slots + fixed::kVjpU + 4 * i + a, &q.u[a][i], 8);
+      std::memcpy(slots + fixed::kVjpU + 12 + a, &q.p[a], 8);
+      for (int i = 0; i < 4; ++i) std::memcpy(slots + fixed::kVjpW + 4 * i + a, &q.w[a][i], 8);
+    }
+    if (!fixed::element_vjp_fixed<FLAGS, 1>({slots, words}, q.inv, q.rh, FP,
+                                            [&](int i, int a) { return q.u[a][i]; }, Keep{G}))
+      ++left;
+    const ld step = 1e-30L;
+    for (int b = 0; b < 4; ++b)
+      for (int k = 0; k < 4; ++k) {
+        cld u[4][3], p[4], F[4][4];
+        for (int a = 0; a < 4; ++a) {
+          for (int i = 0; i < 3; ++i) u[a][i] = cld(q.u[a][i], a == b && i == k ? step : 0);
+          p[a] = cld(q.p[a], a == b && k == 3 ? step : 0);
+        }
+        reference<FLAGS, cld>(q.X, u, p, q.P, F);
+        ld r = 0;
+        for (int a = 0; a < 4; ++a)
+          for (int i = 0; i < 4; ++i) r += q.w[a][i] * (F[a][i].imag() / step);
+        const double mine = k < 3 ? gu[b][k] : gp[b];
+        e[k] += std::pow((double)(G[b][k] - r), 2);
+        d[k] += std::pow((double)(mine - r), 2);
+        norm[k] += std::pow((double)r, 2);
+      }
+  }
+  say("left_vjp", FLAGS, kind, left, 0);
+  for (int k = 0; k < 4; ++k)
+    say(k < 3 ? "velocity_grad" : "pressure_grad", FLAGS, kind, std::sqrt(e[k] / norm[k]),
+        1.1 * std::sqrt(d[k] / norm[k]));
+}
 template <int FLAGS>
 static void routines(int n) {
   // the eddy viscosity of kinds 2 and 3 is ill-conditioned in any arithmetic
   for (int kind : {0, 1, 2, 3, 4, 5})
     if (!(FLAGS & kVreman) || kind < 2 || kind > 3) routine<FLAGS>(kind, n);
+  for (int kind : {0, 1, 2, 3})
+    if (!(FLAGS & kVreman) || kind < 2) adjoint<FLAGS>(kind, n / 4);
 }
 
 // Data outside the range leave the routine before it has written anything.
