@@ -60,17 +60,17 @@ constexpr int64_t kQB61 = 0x46c1b47480244d9ll;          // QB 2^61
 constexpr int64_t kEightFifteenths60 = 0x888888888888889ll;  // (8/15) 2^60
 constexpr int64_t kTwoThirds61 = 0x1555555555555555ll;  // (2/3) 2^61; 1/24 = 2^-4 2/3
 
-// Per-thread scratch in shared memory: 64-bit slots and 32-bit words, the
-// same slot of the block's THREADS threads side by side (no bank conflicts).
-// Rolled loops index it at run time.
+// Per-thread scratch in shared memory: 64-bit slots and 16-bit words (for
+// exponents), the same slot of the block's THREADS threads side by side (no
+// bank conflicts). Rolled loops index it at run time.
 constexpr int kFwdSlots = 49;   // 64-bit slots of element_rhs_fixed
 constexpr int kFwdSlotsSkew = 61;
-constexpr int kFwdWords = 15;   // 32-bit words
+constexpr int kFwdWords = 15;   // 16-bit words
 
 template <int THREADS>
 struct Scratch {
   int64_t* q;  // + threadIdx.x
-  int32_t* w;
+  int16_t* w;
   __device__ __forceinline__ int64_t get(int s) const { return q[s * THREADS]; }
   __device__ __forceinline__ void put(int s, int64_t x) const { q[s * THREADS] = x; }
   __device__ __forceinline__ Limb limb(int s) const {
@@ -85,7 +85,7 @@ struct Scratch {
     q[s * THREADS] = (int64_t)((uint64_t)(uint32_t)hi_word(x) << 32 | lo_word(x));
   }
   __device__ __forceinline__ int32_t word(int s) const { return w[s * THREADS]; }
-  __device__ __forceinline__ void put_word(int s, int32_t x) const { w[s * THREADS] = x; }
+  __device__ __forceinline__ void put_word(int s, int32_t x) const { w[s * THREADS] = (int16_t)x; }
 };
 
 // Slots. C: cofactors (input c_k,j, k = 1..3, at kSlotC + 3 (k - 1) + j, then

@@ -16,12 +16,16 @@
 namespace nsrhs {
 namespace fixed {
 
-// Slots of element_vjp_fixed. C: as in the forward, then tau and k2/|u_g| of
-// the Gauss points. U: nodal values of component i (u, v, w, p) of node a at
-// kVjpU + 4 i + a, then W~. X: tau W~ from the pressure's input slots on, then
-// the Gauss points' gradients. W: the cotangent, component i of node a at
-// kVjpW + 4 i + a. R: gradient rows of u, v, w, p and of the cotangent.
-enum : int { kVjpC = 0, kVjpU = 9, kVjpX = 21, kVjpW = 33, kVjpR = 49, kVjpSlots = 73 };
+// Slots of element_vjp_fixed, laid over one another so that 12 warps share
+// an SM. U: velocities, component i of node a at kVjpU + 4 i + a; then W, W~
+// and back to u. X: cofactors (input c_k,j at kVjpC + 3 (k - 1) + j, then
+// limbs); then the contractions for the Gauss points, tau and k2/|u_g|, and the
+// Gauss points' gradients. W: the cotangent, component i of node a at kVjpW +
+// 4 i + a; the slots of its component 3 end as a row's four sums. R: gradient
+// rows of u, v, w, p and of the cotangent; the pressure's input values lie in
+// the last four until its row is made, the pressure's row ends as scratch.
+enum : int { kVjpU = 0, kVjpX = 12, kVjpC = kVjpX + 3, kVjpW = 24, kVjpR = 40, kVjpSlots = 64 };
+enum : int { kVjpP = kVjpR + 20, kVjpY = kVjpW + 12, kVjpK = kVjpR + 9 };
 enum : int { kVjpT = 0, kVjpEu = 3, kVjpEg = 11, kVjpXg = 19, kVjpWords = 23 };
 
 // raw(i, a): component i of the velocity at node a as the caller's double.
@@ -58,7 +62,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
   // gradient rows (real R 2^(eg_i + t_j - 61)), W of the velocities ----
 #pragma unroll 1
   for (int i = 0; i < 8; ++i) {
-    const int at = i < 4 ? kVjpU + 4 * i : kVjpW + 4 * (i - 4);
+    const int at = i < 3 ? kVjpU + 4 * i : i == 3 ? kVjpP : kVjpW + 4 * (i - 4);
     double u[4];
 #pragma unroll
     for (int a = 0; a < 4; ++a) u[a] = sc.real(at + a);
@@ -109,123 +113,11 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
   const int kap = imax(eu[0] + t[0], imax(eu[1] + t[1], eu[2] + t[2]));
   auto row = [&](int i, int j) { return sc.get(kVjpR + 3 * i + j); };
 
-  // ---- viscosity ----
-  double mu_eff = P.P.mu;
-  double vA = 0.0, vphi = 0.0, vscale = 0.0;
-  bool vactive = false;
-  if constexpr (VREMAN) {
-    double g[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) g[i][j] = to_double(row(i, j), eG[i] + t[j] - 1);
-    vreman_viscosity(g, rh, P, vA, vphi, vscale, mu_eff, vactive);
-  }
-  const double rh2 = rh * rh;
-  const double k1 = (VREMAN ? P.P.c1 * mu_eff : P.c1mu) * rh2;
-
-  double stau = 0.0, tau_e = 0.0, yr_e = 0.0;
-  double S[3] = {0.0, 0.0, 0.0};  // sum of the nodal velocities
-  const double k2 = P.k2 * rh;
-  int ete = 0;
-  int64_t tme = 0;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) S[i] = (raw(i, 0) + raw(i, 1)) + (raw(i, 2) + raw(i, 3));
-  if constexpr (TAUE) {
-    const double sm = fmac(S[2], S[2], fmac(S[1], S[1], S[0] * S[0])) * 0.0625;
-    yr_e = M::rsqrt_(sm);
-    tau_e = M::rcp(fmac(k2, sm * yr_e, k1));
-    stau = 4.0 * tau_e;
-    tme = scalar_fixed(tau_e, ete);
-  }
-
-  // ---- per Gauss point: tau_g and k2 / |u_g|, W~, tau W~ ----
-  const double k2a = P.k2a * rh;
-  int theta = -32768;
-#pragma unroll 1
-  for (int g = 0; g < 4; ++g) {
-    int64_t w[3];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) w[j] = sc.get(kVjpU + 4 * j + g);
-    int et = ete;
-    int64_t tm = tme;
-    if constexpr (!TAUE) {
-      const double s = velocity_norm2(w[0], w[1], w[2], eu, eum);  // |u_g|^2 / alpha^2
-      const double y = k2a * M::rsqrt_(s);                         // alpha^2 k2 / |u_g|
-      const double tau = M::rcp(fmac(y, s, k1));
-      sc.put_real(kVjpC + g, tau);
-      sc.put_real(kVjpC + 4 + g, y * 5.0);  // alpha^2 = 1/5
-      stau += tau;
-      tm = scalar_fixed(tau, et);
-    }
-    const Limb tl = limb(tm);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      w[j] = shr(w[j], kap - (eu[j] + t[j]));
-      sc.put(kVjpU + 4 * j + g, limb(w[j]));
-    }
-    const int n = norm_shift(mag(w[0]) | mag(w[1]) | mag(w[2]));
-    sc.put_word(kVjpXg + g, et - n);
-    theta = imax(theta, et - n);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) sc.put(kVjpX + 3 * g + j, mul8(tl, limb(shl(w[j], n))));
-  }
-
-  // ---- T, Q; Qp = a2 Q + a1 I, sT = b4 T ----
-  Limb Qp[6], sT[3];
-  int eP, eT;
-  int einv;
-  const Limb inv = limb(scalar_fixed(inv_det, einv));
-  {
-    int64_t Tc[3] = {0, 0, 0}, V[3] = {0, 0, 0};
-    Acc q[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) q[k] = acc_start();
-#pragma unroll 1
-    for (int g = 0; g < 4; ++g) {
-      const int k = theta - sc.word(kVjpXg + g);
-      Limb v[3], w[3];
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const int64_t y = shr(sc.get(kVjpX + 3 * g + j), k);
-        Tc[j] += y;
-        v[j] = limb(y);
-        w[j] = sc.limb(kVjpU + 4 * j + g);
-        V[j] += whole(w[j]);
-      }
-      mac(q[0], v[0], w[0]);
-      mac(q[1], v[1], w[1]);
-      mac(q[2], v[2], w[2]);
-      mac(q[3], v[0], w[1]);
-      mac(q[4], v[0], w[2]);
-      mac(q[5], v[1], w[2]);
-    }
-    Limb a1l = P.a1.m;
-    int ea1 = P.a1.e + einv;
-    if constexpr (VREMAN) {
-      if (vactive) {
-        int em;
-        const Limb mm = limb(scalar_fixed(mu_eff, em));
-        a1l = limb(mul8(mm, nsrhs::fixed::limb(-kTwoThirds61)) * 2);
-        ea1 = em - 2 + einv;
-      }
-    }
-    gauss_matrices(q, Tc, theta, kap, inv, einv, mul8(inv, a1l), ea1, t, tmax, P, Qp, eP, sT, eT);
-    // W~_a back to u_a = W_a - QB sum_b W_b (the sum is S sqrt 5)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) V[j] = qb_sum(V[j]);
-#pragma unroll 1
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-        sc.put(kVjpU + 4 * j + a, limb(whole(sc.limb(kVjpU + 4 * j + a)) - V[j]));
-  }
-
-  // ---- FP64: reverse sweep at the Gauss points ----
+  // ---- contractions for the reverse sweep at the Gauss points ----
   const double s24 = inv_det * (1.0 / 24.0);
   double mub = 0.0;   // mu_eff-bar (used with the eddy viscosity)
+  double Qh[3][3], Tb[3], staub;
   {
-    double Qh[3][3], Tb[3], staub;
     // Qh = (a2 / 2) (G^T Om + Om^T G): the component index aligned through G
     {
       const int e[3] = {eG[0] + eO[0], eG[1] + eO[1], eG[2] + eO[2]};
@@ -285,6 +177,123 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
       Qh[0][2] = Qh[2][0] = a2 * x[4];
       Qh[1][2] = Qh[2][1] = a2 * x[5];
     }
+  }
+
+  // ---- viscosity ----
+  double mu_eff = P.P.mu;
+  double vA = 0.0, vphi = 0.0, vscale = 0.0;
+  bool vactive = false;
+  if constexpr (VREMAN) {
+    double g[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) g[i][j] = to_double(row(i, j), eG[i] + t[j] - 1);
+    vreman_viscosity(g, rh, P, vA, vphi, vscale, mu_eff, vactive);
+  }
+  const double rh2 = rh * rh;
+  const double k1 = (VREMAN ? P.P.c1 * mu_eff : P.c1mu) * rh2;
+
+  double stau = 0.0, tau_e = 0.0, yr_e = 0.0;
+  double S[3] = {0.0, 0.0, 0.0};  // sum of the nodal velocities
+  const double k2 = P.k2 * rh;
+  int ete = 0;
+  int64_t tme = 0;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) S[i] = (raw(i, 0) + raw(i, 1)) + (raw(i, 2) + raw(i, 3));
+  if constexpr (TAUE) {
+    const double sm = fmac(S[2], S[2], fmac(S[1], S[1], S[0] * S[0])) * 0.0625;
+    yr_e = M::rsqrt_(sm);
+    tau_e = M::rcp(fmac(k2, sm * yr_e, k1));
+    stau = 4.0 * tau_e;
+    tme = scalar_fixed(tau_e, ete);
+  }
+
+  // ---- per Gauss point: tau_g and k2 / |u_g|, W~, tau W~ ----
+  const double k2a = P.k2a * rh;
+  int theta = -32768;
+#pragma unroll 1
+  for (int g = 0; g < 4; ++g) {
+    int64_t w[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) w[j] = sc.get(kVjpU + 4 * j + g);
+    int et = ete;
+    if constexpr (!TAUE) {
+      const double s = velocity_norm2(w[0], w[1], w[2], eu, eum);  // |u_g|^2 / alpha^2
+      const double y = k2a * M::rsqrt_(s);                         // alpha^2 k2 / |u_g|
+      const double tau = M::rcp(fmac(y, s, k1));
+      sc.put_real(kVjpX + 3 * g, tau);
+      sc.put_real(kVjpX + 3 * g + 1, y * 5.0);  // alpha^2 = 1/5
+      stau += tau;
+      et = scalar_exp(tau);
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      w[j] = shr(w[j], kap - (eu[j] + t[j]));
+      sc.put(kVjpU + 4 * j + g, limb(w[j]));
+    }
+    const int n = norm_shift(mag(w[0]) | mag(w[1]) | mag(w[2]));
+    sc.put_word(kVjpXg + g, n);
+    theta = imax(theta, et - n);
+  }
+
+  // ---- T, Q; Qp = a2 Q + a1 I, sT = b4 T ----
+  Limb Qp[6], sT[3];
+  int eP, eT;
+  int einv;
+  const Limb inv = limb(scalar_fixed(inv_det, einv));
+  {
+    int64_t Tc[3] = {0, 0, 0}, V[3] = {0, 0, 0};
+    Acc q[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) q[k] = acc_start();
+#pragma unroll 1
+    for (int g = 0; g < 4; ++g) {
+      // tau W~ from the normalised W~, real 2^(et - n + kap - t_j - 58)
+      int et = ete;
+      int64_t tm = tme;
+      if constexpr (!TAUE) tm = scalar_fixed(sc.real(kVjpX + 3 * g), et);
+      const Limb tl = limb(tm);
+      const int n = sc.word(kVjpXg + g), k = theta - (et - n);
+      Limb v[3], w[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        w[j] = sc.limb(kVjpU + 4 * j + g);
+        const int64_t x = whole(w[j]), y = shr(mul8(tl, limb(shl(x, n))), k);
+        Tc[j] += y;
+        v[j] = limb(y);
+        V[j] += x;
+      }
+      mac(q[0], v[0], w[0]);
+      mac(q[1], v[1], w[1]);
+      mac(q[2], v[2], w[2]);
+      mac(q[3], v[0], w[1]);
+      mac(q[4], v[0], w[2]);
+      mac(q[5], v[1], w[2]);
+    }
+    Limb a1l = P.a1.m;
+    int ea1 = P.a1.e + einv;
+    if constexpr (VREMAN) {
+      if (vactive) {
+        int em;
+        const Limb mm = limb(scalar_fixed(mu_eff, em));
+        a1l = limb(mul8(mm, nsrhs::fixed::limb(-kTwoThirds61)) * 2);
+        ea1 = em - 2 + einv;
+      }
+    }
+    gauss_matrices(q, Tc, theta, kap, inv, einv, mul8(inv, a1l), ea1, t, tmax, P, Qp, eP, sT, eT);
+    // W~_a back to u_a = W_a - QB sum_b W_b (the sum is S sqrt 5)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) V[j] = qb_sum(V[j]);
+#pragma unroll 1
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        sc.put(kVjpU + 4 * j + a, limb(whole(sc.limb(kVjpU + 4 * j + a)) - V[j]));
+  }
+
+  // ---- FP64: reverse sweep at the Gauss points ----
+  {
     double Os[3][3];
     if constexpr (SKEW) {
       const double r48 = P.P.rho * (1.0 / 48.0);
@@ -327,7 +336,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
 #pragma unroll
       for (int i = 0; i < 3; ++i) ug[i] = fmac(kQA - kQB, raw(i, g), bS[i]);
       if constexpr (!TAUE) {
-        const double tau = sc.real(kVjpC + g), kyr = sc.real(kVjpC + 4 + g);
+        const double tau = sc.real(kVjpX + 3 * g), kyr = sc.real(kVjpX + 3 * g + 1);
         double QT[3];
 #pragma unroll
         for (int i = 0; i < 3; ++i)
@@ -429,7 +438,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
         const int64_t h = shr(mul8(P.m120.m, limb(sc.get(kVjpR + 3 * k + i))),
                               eF - (eh + sc.word(kVjpEg + k) + sc.word(kVjpEu + 4 + k)));
         mh |= mag(h);
-        sc.put(kVjpC + 4 + k, h);
+        sc.put(kVjpK + k, h);
       }
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
@@ -444,7 +453,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
         Kl[j] = limb(shl(K[j], n));
-        Hl[j] = limb(shl(sc.get(kVjpC + 4 + j), n));
+        Hl[j] = limb(shl(sc.get(kVjpK + j), n));
       }
       base = 0;
       e = eF - n + 5;
@@ -454,7 +463,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
       const int64_t sm = scalar_fixed(stau, es);
       const Limb sg = limb(mul8(limb(mul8(inv, nsrhs::fixed::limb(-kTwoThirds61))), limb(sm * 2)));
       e = trace_row(sc, kVjpR + 12, kVjpR + 21, kVjpEg + 4, kVjpT, eO, t, tmax, sT, eT, sg, einv - 4 + es + ecw,
-                    kTwoThirds61 / 2, kVjpC + 4, Kl, base);
+                    kTwoThirds61 / 2, kVjpK, Kl, base);
     }
     int64_t y[4];
     y[0] = base;
@@ -465,10 +474,10 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
       y[a] += base;
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a) sc.put(kVjpC + a, y[a]);
+    for (int a = 0; a < 4; ++a) sc.put(kVjpY + a, y[a]);
 #pragma unroll 1
     for (int a = 0; a < 4; ++a) {
-      int64_t z = sc.get(kVjpC + a);
+      int64_t z = sc.get(kVjpY + a);
       double x = 0.0;
       if (i < 3) {
         z = dot3(Hl[0], limb(sc.get(kVjpW + a)), Hl[1], limb(sc.get(kVjpW + 4 + a)), Hl[2],

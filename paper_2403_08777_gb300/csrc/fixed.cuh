@@ -110,8 +110,9 @@ __device__ __forceinline__ int64_t to_fixed(double x, int E) {
   return hi < 0 ? -a : a;
 }
 
-// Mantissa in [2^59, 2^60) and exponent of a positive normal double:
+// Exponent of a positive normal double, and its mantissa in [2^59, 2^60):
 // x = result 2^(e - 60).
+__device__ __forceinline__ int scalar_exp(double x) { return ((hi_word(x) >> 20) & 0x7ff) - 1022; }
 __device__ __forceinline__ int64_t scalar_fixed(double x, int& e) {
   const int32_t hi = hi_word(x);
   e = ((hi >> 20) & 0x7ff) - 1022;

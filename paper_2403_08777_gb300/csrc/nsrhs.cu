@@ -464,8 +464,8 @@ __device__ __forceinline__ void load_geometry(const R* __restrict__ geom, int64_
 // the per-mesh cache (an 88-byte streamed record), or the node coordinates
 // gathered through the connectivity and formed into the Jacobian in the
 // call itself (Sec. V-B's per-element constant gradients, 43 FP64 operations).
-// get(): into registers; stage(): the cofactors into the scratch slots of the
-// fixed-point routines, 1/detJ and detJ^(-1/3) into registers.
+// get(): into registers; stage(): the cofactors into the scratch slots from
+// `at` on, 1/detJ and detJ^(-1/3) into registers.
 struct GeomCached {
   const double* __restrict__ geom;
   __device__ __forceinline__ void get(int64_t E, int64_t e, const int32_t v[4], double c[3][3],
@@ -473,11 +473,11 @@ struct GeomCached {
     load_geometry(geom, E, e, c, inv_det, rh);
   }
   template <int T>
-  __device__ __forceinline__ void stage(const nsrhs::fixed::Scratch<T>& sc, int64_t E, int64_t e,
-                                        const int32_t v[4], double& inv_det, double& rh) const {
-    static_assert(nsrhs::fixed::kSlotC == 0 && nsrhs::fixed::kVjpC == 0, "cofactor slots");
+  __device__ __forceinline__ void stage(const nsrhs::fixed::Scratch<T>& sc, int at, int64_t E,
+                                        int64_t e, const int32_t v[4], double& inv_det,
+                                        double& rh) const {
 #pragma unroll
-    for (int q = 0; q < 9; ++q) nsrhs::cp_async<8>(sc.q + q * T, geom + q * E + e);
+    for (int q = 0; q < 9; ++q) nsrhs::cp_async<8>(sc.q + (at + q) * T, geom + q * E + e);
     inv_det = ldg(geom + 9 * E + e);
     rh = ldg(geom + 10 * E + e);
   }
@@ -495,12 +495,13 @@ struct GeomRecompute {
     nsrhs::element_geometry<double, double>(X, c, inv_det, rh);
   }
   template <int T>
-  __device__ __forceinline__ void stage(const nsrhs::fixed::Scratch<T>& sc, int64_t E, int64_t e,
-                                        const int32_t v[4], double& inv_det, double& rh) const {
+  __device__ __forceinline__ void stage(const nsrhs::fixed::Scratch<T>& sc, int at, int64_t E,
+                                        int64_t e, const int32_t v[4], double& inv_det,
+                                        double& rh) const {
     double c[3][3];
     get(E, e, v, c, inv_det, rh);
 #pragma unroll
-    for (int q = 0; q < 9; ++q) sc.put_real(q, c[q / 3][q % 3]);
+    for (int q = 0; q < 9; ++q) sc.put_real(at + q, c[q / 3][q % 3]);
   }
 };
 
@@ -553,7 +554,7 @@ struct AddEntries {
 };
 
 // The double-precision kernels run one warp per CTA: their scratch in shared
-// memory (14 KB a warp) and 128 registers let 15 warps share an SM, and a
+// memory (13 KB a warp) and 128 registers let 16 warps share an SM, and a
 // small mesh spreads over as many SMs as it has warps. 64 and 128 threads
 // per CTA measured the same on large meshes (128^3: 2.79, 2.79, 2.91 ms).
 constexpr int kFixedThreads = 32;
@@ -567,14 +568,14 @@ constexpr int kFixedThreads = 32;
 // fixes the summation order (bitwise reproducible).
 //
 // Bound by instruction issue (ALU pipe 60 % busy, 4650 instructions a warp at
-// 0.53 per clock and sub-partition), where the FP64 form kept the FP64 pipe
+// 0.55 per clock and sub-partition), where the FP64 form kept the FP64 pipe
 // 90 % busy with 344 FP64 instructions (64 clocks of a sub-partition each):
-// 256^3 61.3 -> 22.7 ms.
+// 256^3 61.3 -> 21.9 ms.
 //
 // plain: every element on the FP64 pipe (parameters outside the fixed-point
 // range).
 template <int FLAGS, class GS>
-__global__ void __launch_bounds__(kFixedThreads, 15)
+__global__ void __launch_bounds__(kFixedThreads, 16)
     fwd_fp64_kernel(int64_t N, int64_t E, int64_t e0, int64_t e1,
                     const int32_t* __restrict__ conn, GS gs, const double* __restrict__ up,
                     const __grid_constant__ FixedParams P, bool plain,
@@ -583,7 +584,7 @@ __global__ void __launch_bounds__(kFixedThreads, 15)
   constexpr int T = kFixedThreads;
   constexpr int slots = (FLAGS & nsrhs::kSkew) ? fx::kFwdSlotsSkew : fx::kFwdSlots;
   __shared__ int64_t sq[slots * T];
-  __shared__ int32_t sw[fx::kFwdWords * T];
+  __shared__ int16_t sw[fx::kFwdWords * T];
   const fx::Scratch<T> sc{sq + threadIdx.x, sw + threadIdx.x};
   for (int64_t e = e0 + blockIdx.x * (int64_t)T + threadIdx.x; e < e1; e += (int64_t)gridDim.x * T) {
     if (!plain) {
@@ -596,7 +597,7 @@ __global__ void __launch_bounds__(kFixedThreads, 15)
         for (int i = 0; i < 4; ++i)
           nsrhs::cp_async<8>(sc.q + (fx::kSlotU + 4 * i + a) * T, up + i * N + v[a]);
       double inv_det, rh;
-      gs.stage(sc, E, e, v, inv_det, rh);
+      gs.stage(sc, fx::kSlotC, E, e, v, inv_det, rh);
       nsrhs::cp_async_commit();
       nsrhs::cp_async_wait<0>();
       if (fx::element_rhs_fixed<FLAGS, T>(sc, inv_det, rh, P, AddEntries{rhs, N, v})) continue;
@@ -735,12 +736,14 @@ struct NodalVelocity {
 
 // FP64 adjoint of the elements [e0, e1) (row stride E), one per thread; the
 // two uses, GS and plain as in fwd_fp64_kernel. Integer and FP64 pipe share
-// the sweep (element_fixed_vjp.cuh): FP64 pipe 60 % busy, ALU 37 %, 0.38
-// instructions per clock and sub-partition with the 10 warps per SM that
-// 22 KB of scratch a warp allow, where the FP64 form kept the FP64 pipe 90 %
-// busy with 648 instructions: 256^3 114.4 -> 60.5 ms.
+// the sweep (element_fixed_vjp.cuh): FP64 pipe 65 % busy, ALU 41 %. A warp's
+// instructions wait on one another (6.6 clocks each), so the time falls with
+// the warps that share an SM: 12 with 18 KB of scratch a warp, where slots are
+// laid over one another and tau W~ is formed twice rather than kept; 10 with
+// 22 KB took 128^3 7.67 ms, 12 take 7.08 ms. The FP64 form kept the FP64 pipe
+// 90 % busy with 648 instructions: 256^3 114.4 ms.
 template <int FLAGS, class GS>
-__global__ void __launch_bounds__(kFixedThreads, 10)
+__global__ void __launch_bounds__(kFixedThreads, 12)
     vjp_fp64_kernel(int64_t N, int64_t E, int64_t e0, int64_t e1,
                     const int32_t* __restrict__ conn, GS gs, const double* __restrict__ up,
                     const double* __restrict__ cot, const __grid_constant__ FixedParams P,
@@ -748,7 +751,7 @@ __global__ void __launch_bounds__(kFixedThreads, 10)
   namespace fx = nsrhs::fixed;
   constexpr int T = kFixedThreads;
   __shared__ int64_t sq[fx::kVjpSlots * T];
-  __shared__ int32_t sw[fx::kVjpWords * T];
+  __shared__ int16_t sw[fx::kVjpWords * T];
   const fx::Scratch<T> sc{sq + threadIdx.x, sw + threadIdx.x};
   for (int64_t e = e0 + blockIdx.x * (int64_t)T + threadIdx.x; e < e1; e += (int64_t)gridDim.x * T) {
     if (!plain) {
@@ -759,11 +762,12 @@ __global__ void __launch_bounds__(kFixedThreads, 10)
       for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          nsrhs::cp_async<8>(sc.q + (fx::kVjpU + 4 * i + a) * T, up + i * N + v[a]);
+          nsrhs::cp_async<8>(sc.q + (i < 3 ? fx::kVjpU + 4 * i + a : fx::kVjpP + a) * T,
+                             up + i * N + v[a]);
           nsrhs::cp_async<8>(sc.q + (fx::kVjpW + 4 * i + a) * T, cot + i * N + v[a]);
         }
       double inv_det, rh;
-      gs.stage(sc, E, e, v, inv_det, rh);
+      gs.stage(sc, fx::kVjpC, E, e, v, inv_det, rh);
       nsrhs::cp_async_commit();
       nsrhs::cp_async_wait<0>();
       if (fx::element_vjp_fixed<FLAGS, T>(sc, inv_det, rh, P, NodalVelocity{up, N, v},
@@ -973,7 +977,7 @@ FixedParams fixed_params(const nsrhs_params* p) {
   return nsrhs::fixed::make_fixed_params(elem_params<double>(p), p->convection == NSRHS_SKEW);
 }
 
-// Grid of a one-warp-per-CTA kernel over n elements: several waves of the 15
+// Grid of a one-warp-per-CTA kernel over n elements: several waves of the 16
 // resident CTAs per SM.
 unsigned fixed_grid(int64_t n, int device) {
   const int64_t need = (n + kFixedThreads - 1) / kFixedThreads;

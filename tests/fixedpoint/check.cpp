@@ -222,7 +222,7 @@ static void routine(int kind, int n) {
     double F[4][4], G[4][4];
     element_rhs<double, FLAGS>(q.c, q.inv, q.rh, q.u, q.p, q.P, F);
     int64_t slots[128];
-    int32_t words[32];
+    int16_t words[32];
     stage(q, slots);
     if (!fixed::element_rhs_fixed<FLAGS, 1>({slots, words}, q.inv, q.rh, FP, Keep{G})) ++left;
     ld u[4][3], p[4], R[4][4];
@@ -256,11 +256,11 @@ static void adjoint(int kind, int n) {
     double gu[4][3], gp[4], G[4][4];
     element_vjp<double, FLAGS>(q.c, q.inv, q.rh, q.u, q.p, q.w, q.P, gu, gp);
     int64_t slots[128];
-    int32_t words[32];
+    int16_t words[32];
     for (int k = 0; k < 9; ++k) std::memcpy(slots + fixed::kVjpC + k, &q.c[k / 3][k % 3], 8);
     for (int a = 0; a < 4; ++a) {
       for (int i = 0; i < 3; ++i) std::memcpy(slots + fixed::kVjpU + 4 * i + a, &q.u[a][i], 8);
-      std::memcpy(slots + fixed::kVjpU + 12 + a, &q.p[a], 8);
+      std::memcpy(slots + fixed::kVjpP + a, &q.p[a], 8);
       for (int i = 0; i < 4; ++i) std::memcpy(slots + fixed::kVjpW + 4 * i + a, &q.w[a][i], 8);
     }
     if (!fixed::element_vjp_fixed<FLAGS, 1>({slots, words}, q.inv, q.rh, FP,
@@ -315,7 +315,7 @@ static void range() {
       if (at == 7) q.inv = std::fabs(x) == 0x1p-1074 ? 1e-300 : x == 1e40 || x == -1e40 || x == 1e-40 ? INFINITY : x;
       if (x == 0x1p-1074 && at < 7) continue;  // subnormal data count as 0
       int64_t slots[128];
-      int32_t words[32];
+      int16_t words[32];
       stage(q, slots);
       const auto FP = fixed::make_fixed_params(q.P, false);
       if (fixed::element_rhs_fixed<0, 1>({slots, words}, q.inv, q.rh, FP, Never{&calls})) ++bad;
