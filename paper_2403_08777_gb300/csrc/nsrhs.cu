@@ -570,7 +570,7 @@ constexpr int kFixedThreads = 32;
 // Bound by instruction issue (ALU pipe 60 % busy, 4650 instructions a warp at
 // 0.55 per clock and sub-partition), where the FP64 form kept the FP64 pipe
 // 90 % busy with 344 FP64 instructions (64 clocks of a sub-partition each):
-// 256^3 61.3 -> 21.9 ms.
+// 256^3 61.3 -> 20.5 ms.
 //
 // plain: every element on the FP64 pipe (parameters outside the fixed-point
 // range).
@@ -586,24 +586,24 @@ __global__ void __launch_bounds__(kFixedThreads, 16)
   __shared__ int64_t sq[slots * T];
   __shared__ int16_t sw[fx::kFwdWords * T];
   const fx::Scratch<T> sc{sq + threadIdx.x, sw + threadIdx.x};
-  for (int64_t e = e0 + blockIdx.x * (int64_t)T + threadIdx.x; e < e1; e += (int64_t)gridDim.x * T) {
-    if (!plain) {
-      int32_t v[4];
+  const int64_t e = e0 + blockIdx.x * (int64_t)T + threadIdx.x;
+  if (e >= e1) return;
+  if (!plain) {
+    int32_t v[4];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) v[a] = ldg(conn + a * E + e);
+    for (int a = 0; a < 4; ++a) v[a] = ldg(conn + a * E + e);
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          nsrhs::cp_async<8>(sc.q + (fx::kSlotU + 4 * i + a) * T, up + i * N + v[a]);
-      double inv_det, rh;
-      gs.stage(sc, fx::kSlotC, E, e, v, inv_det, rh);
-      nsrhs::cp_async_commit();
-      nsrhs::cp_async_wait<0>();
-      if (fx::element_rhs_fixed<FLAGS, T>(sc, inv_det, rh, P, AddEntries{rhs, N, v})) continue;
-    }
-    fwd_fp64_plain<FLAGS, GS>(N, E, e, conn, gs, up, P.P, rhs);
+      for (int i = 0; i < 4; ++i)
+        nsrhs::cp_async<8>(sc.q + (fx::kSlotU + 4 * i + a) * T, up + i * N + v[a]);
+    double inv_det, rh;
+    gs.stage(sc, fx::kSlotC, E, e, v, inv_det, rh);
+    nsrhs::cp_async_commit();
+    nsrhs::cp_async_wait<0>();
+    if (fx::element_rhs_fixed<FLAGS, T>(sc, inv_det, rh, P, AddEntries{rhs, N, v})) return;
   }
+  fwd_fp64_plain<FLAGS, GS>(N, E, e, conn, gs, up, P.P, rhs);
 }
 
 // Element-matrix comparison kernel: the same RHS through a full 16x16
@@ -741,7 +741,7 @@ struct NodalVelocity {
 // the warps that share an SM: 12 with 18 KB of scratch a warp, where slots are
 // laid over one another and tau W~ is formed twice rather than kept; 10 with
 // 22 KB took 128^3 7.67 ms, 12 take 7.08 ms. The FP64 form kept the FP64 pipe
-// 90 % busy with 648 instructions: 256^3 114.4 ms.
+// 90 % busy with 648 instructions: 256^3 114.4 -> 52.2 ms.
 template <int FLAGS, class GS>
 __global__ void __launch_bounds__(kFixedThreads, 12)
     vjp_fp64_kernel(int64_t N, int64_t E, int64_t e0, int64_t e1,
@@ -753,29 +753,29 @@ __global__ void __launch_bounds__(kFixedThreads, 12)
   __shared__ int64_t sq[fx::kVjpSlots * T];
   __shared__ int16_t sw[fx::kVjpWords * T];
   const fx::Scratch<T> sc{sq + threadIdx.x, sw + threadIdx.x};
-  for (int64_t e = e0 + blockIdx.x * (int64_t)T + threadIdx.x; e < e1; e += (int64_t)gridDim.x * T) {
-    if (!plain) {
-      int32_t v[4];
+  const int64_t e = e0 + blockIdx.x * (int64_t)T + threadIdx.x;
+  if (e >= e1) return;
+  if (!plain) {
+    int32_t v[4];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) v[a] = ldg(conn + a * E + e);
+    for (int a = 0; a < 4; ++a) v[a] = ldg(conn + a * E + e);
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          nsrhs::cp_async<8>(sc.q + (i < 3 ? fx::kVjpU + 4 * i + a : fx::kVjpP + a) * T,
-                             up + i * N + v[a]);
-          nsrhs::cp_async<8>(sc.q + (fx::kVjpW + 4 * i + a) * T, cot + i * N + v[a]);
-        }
-      double inv_det, rh;
-      gs.stage(sc, fx::kVjpC, E, e, v, inv_det, rh);
-      nsrhs::cp_async_commit();
-      nsrhs::cp_async_wait<0>();
-      if (fx::element_vjp_fixed<FLAGS, T>(sc, inv_det, rh, P, NodalVelocity{up, N, v},
-                                          AddEntries{grad, N, v}))
-        continue;
-    }
-    vjp_fp64_plain<FLAGS, GS>(N, E, e, conn, gs, up, cot, P.P, grad);
+      for (int i = 0; i < 4; ++i) {
+        nsrhs::cp_async<8>(sc.q + (i < 3 ? fx::kVjpU + 4 * i + a : fx::kVjpP + a) * T,
+                           up + i * N + v[a]);
+        nsrhs::cp_async<8>(sc.q + (fx::kVjpW + 4 * i + a) * T, cot + i * N + v[a]);
+      }
+    double inv_det, rh;
+    gs.stage(sc, fx::kVjpC, E, e, v, inv_det, rh);
+    nsrhs::cp_async_commit();
+    nsrhs::cp_async_wait<0>();
+    if (fx::element_vjp_fixed<FLAGS, T>(sc, inv_det, rh, P, NodalVelocity{up, N, v},
+                                        AddEntries{grad, N, v}))
+      return;
   }
+  vjp_fp64_plain<FLAGS, GS>(N, E, e, conn, gs, up, cot, P.P, grad);
 }
 
 // Mixed-precision vector-Jacobian product of element e: float (u, p), float
@@ -977,11 +977,13 @@ FixedParams fixed_params(const nsrhs_params* p) {
   return nsrhs::fixed::make_fixed_params(elem_params<double>(p), p->convection == NSRHS_SKEW);
 }
 
-// Grid of a one-warp-per-CTA kernel over n elements: several waves of the 16
-// resident CTAs per SM.
-unsigned fixed_grid(int64_t n, int device) {
-  const int64_t need = (n + kFixedThreads - 1) / kFixedThreads;
-  return (unsigned)std::max<int64_t>(1, std::min(need, (int64_t)sm_count(device) * 64));
+// Grid of a one-warp-per-CTA kernel over n elements: one element per thread.
+// An SM takes a new warp when one ends, so the chip stays full to the last
+// wave. With a loop in the kernel and a grid of a few waves the SMs empty at
+// the end of each: 64 CTAs per SM took 2.76 ms for the forward at 128^3 and
+// 7.08 ms for its adjoint, one wave 2.91 and 6.85, this 2.59 and 6.61.
+unsigned fixed_grid(int64_t n) {
+  return (unsigned)std::max<int64_t>(1, (n + kFixedThreads - 1) / kFixedThreads);
 }
 
 template <class R>
@@ -1447,7 +1449,7 @@ nsrhs_status nsrhs_assemble(const nsrhs_mesh* m, const nsrhs_params* p, const vo
     const FixedParams P = fixed_params(p);
     with_flags(flags, [&](auto fl) {
       fwd_fp64_kernel<decltype(fl)::value, GeomRecompute>
-          <<<fixed_grid(E, m->device), kFixedThreads, 0, s>>>(
+          <<<fixed_grid(E), kFixedThreads, 0, s>>>(
               N, E, 0, E, m->conn, GeomRecompute{m->coords, N}, (const double*)up, P,
               !P.in_range, rhs);
     });
@@ -1497,7 +1499,7 @@ nsrhs_status nsrhs_assemble(const nsrhs_mesh* m, const nsrhs_params* p, const vo
         const FixedParams P = fixed_params(p);
         with_flags(flags, [&](auto fl) {
           fwd_fp64_kernel<decltype(fl)::value, GeomCached>
-              <<<fixed_grid(e1 - e0, m->device), kFixedThreads, 0, s>>>(
+              <<<fixed_grid(e1 - e0), kFixedThreads, 0, s>>>(
                   N, E, e0, e1, m->col_conn, GeomCached{m->col_geom}, (const double*)up, P,
                   !P.in_range, rhs);
         });
@@ -1555,7 +1557,7 @@ nsrhs_status nsrhs_assemble(const nsrhs_mesh* m, const nsrhs_params* p, const vo
     const FixedParams P = fixed_params(p);
     with_flags(flags, [&](auto fl) {
       fwd_fp64_kernel<decltype(fl)::value, GeomCached>
-          <<<fixed_grid(E, m->device), kFixedThreads, 0, s>>>(
+          <<<fixed_grid(E), kFixedThreads, 0, s>>>(
               N, E, 0, E, m->conn, GeomCached{m->geom}, (const double*)up, P,
               !P.in_range, rhs);
     });
@@ -1593,7 +1595,7 @@ nsrhs_status nsrhs_assemble_vjp(const nsrhs_mesh* m, const nsrhs_params* p, cons
     const FixedParams P = fixed_params(p);
     with_flags(flags, [&](auto fl) {
       vjp_fp64_kernel<decltype(fl)::value, GeomRecompute>
-          <<<fixed_grid(E, m->device), kFixedThreads, 0, s>>>(
+          <<<fixed_grid(E), kFixedThreads, 0, s>>>(
               N, E, 0, E, m->conn, GeomRecompute{m->coords, N}, (const double*)up,
               (const double*)cot, P, !P.in_range, grad);
     });
@@ -1658,7 +1660,7 @@ nsrhs_status nsrhs_assemble_vjp(const nsrhs_mesh* m, const nsrhs_params* p, cons
         const FixedParams P = fixed_params(p);
         with_flags(formulation_flags(p), [&](auto fl) {
           vjp_fp64_kernel<decltype(fl)::value, GeomCached>
-              <<<fixed_grid(e1 - e0, m->device), kFixedThreads, 0, s>>>(
+              <<<fixed_grid(e1 - e0), kFixedThreads, 0, s>>>(
                   N, E, e0, e1, m->col_conn, GeomCached{m->col_geom}, (const double*)up,
                   (const double*)cot, P, !P.in_range, grad);
         });
@@ -1679,7 +1681,7 @@ nsrhs_status nsrhs_assemble_vjp(const nsrhs_mesh* m, const nsrhs_params* p, cons
     const FixedParams P = fixed_params(p);
     with_flags(formulation_flags(p), [&](auto fl) {
       vjp_fp64_kernel<decltype(fl)::value, GeomCached>
-          <<<fixed_grid(E, m->device), kFixedThreads, 0, s>>>(
+          <<<fixed_grid(E), kFixedThreads, 0, s>>>(
               N, E, 0, E, m->conn, GeomCached{m->geom}, (const double*)up, (const double*)cot, P,
               !P.in_range, grad);
     });
@@ -1766,7 +1768,7 @@ nsrhs_status nsrhs_assemble_rhs_vjp(const nsrhs_mesh* m, const nsrhs_params* p, 
     const FixedParams P = fixed_params(p);
     with_flags(flags, [&](auto fl) {
       constexpr int F = decltype(fl)::value;
-      const unsigned fgrid = fixed_grid(E, m->device);
+      const unsigned fgrid = fixed_grid(E);
       fwd_fp64_kernel<F, GeomCached><<<fgrid, kFixedThreads, 0, s>>>(
           N, E, 0, E, m->conn, GeomCached{m->geom}, (const double*)up, P, !P.in_range, rhs);
       vjp_fp64_kernel<F, GeomCached><<<fgrid, kFixedThreads, 0, s>>>(
