@@ -6,9 +6,12 @@
 // contractions G^T Om, the rows of Gb and their products with the cofactor
 // vectors. They are the bulk of the products, and the rows of Gb and gpb have
 // exactly the form of the forward's momentum and continuity rows.
-// FP64 pipe: tau, and the reverse sweep at the Gauss points, whose terms mix
-// the scaling of gradients and of velocities: about 220 instructions of the
-// FP64 form's 648, beside the integer work.
+// FP64 pipe: tau at the Gauss points, and the reverse sweep there with the
+// eddy viscosity, the skew-symmetric term or the per-element tau. Without
+// these the sweep has integer operands only, and an FP64 instruction costs
+// about five issue slots, so it runs on the integer pipe as well: 256^3 52.2
+// -> 46.3 ms. Its terms mix the scaling of gradients and of velocities; each
+// is normalised by itself, per Gauss point and component, before two meet.
 #pragma once
 
 #include "element_fixed.cuh"
@@ -26,7 +29,7 @@ namespace fixed {
 // the last four until its row is made, the pressure's row ends as scratch.
 enum : int { kVjpU = 0, kVjpX = 12, kVjpC = kVjpX + 3, kVjpW = 24, kVjpR = 40, kVjpSlots = 64 };
 enum : int { kVjpP = kVjpR + 20, kVjpY = kVjpW + 12, kVjpK = kVjpR + 9 };
-enum : int { kVjpT = 0, kVjpEu = 3, kVjpEg = 11, kVjpXg = 19, kVjpWords = 23 };
+enum : int { kVjpT = 0, kVjpEu = 3, kVjpEg = 11, kVjpXg = 19, kVjpWords = 31 };
 
 // raw(i, a): component i of the velocity at node a as the caller's double.
 template <int FLAGS, int THREADS, class Raw, class Out>
@@ -37,6 +40,8 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
   constexpr bool VREMAN = (FLAGS & kVreman) != 0;
   constexpr bool SKEW = (FLAGS & kSkew) != 0;
   constexpr bool TAUE = (FLAGS & kTauElem) != 0;
+  // the reverse sweep at the Gauss points on the integer pipe too
+  constexpr bool INT = FLAGS == 0;
   // ---- cofactor vectors: real C 2^(t_j - 61) ----
   bool ok = (uint32_t)((hi_word(inv_det) >> 20) - 723) <= 600u &&
             (uint32_t)((hi_word(rh) >> 20) - 823) <= 400u;
@@ -115,13 +120,23 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
 
   // ---- contractions for the reverse sweep at the Gauss points ----
   const double s24 = inv_det * (1.0 / 24.0);
+  int einv;
+  const Limb inv = limb(scalar_fixed(inv_det, einv));
   double mub = 0.0;   // mu_eff-bar (used with the eddy viscosity)
   double Qh[3][3], Tb[3], staub;
+  // INT: alpha^2 Qh, with W~ in units 2^(eM + t_j - 60) (see below), alpha Tb in
+  // units 2^(eA + t_j - 60), staub in units 2^(eB - 56)
+  Limb Mq[6];
+  int64_t A[3], st;
+  int eM = 0, eA = 0, eB = 0;
   {
+    uint32_t mx = 0, ma = 0;  // magnitudes of the two contractions
+    int ex = 0, ea = 0;
     // Qh = (a2 / 2) (G^T Om + Om^T G): the component index aligned through G
     {
       const int e[3] = {eG[0] + eO[0], eG[1] + eO[1], eG[2] + eO[2]};
       const int m = imax(e[0], imax(e[1], e[2]));
+      ex = m;
 #pragma unroll 1
       for (int q = 0; q < 6; ++q) {  // entries 00 11 22 01 02 12
         const int j = q < 3 ? q : q == 5 ? 1 : 0, k = q < 3 ? q : q == 3 ? 1 : 2;
@@ -134,9 +149,14 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
           ok_[i] = limb(row(4 + i, k));
         }
         // real 2^(m + t_j + t_k - 59), twice Qh / a2
-        sc.put_real(kVjpX + q, to_double(dot3x<1>(gj[0], ok_[0], gj[1], ok_[1], gj[2], ok_[2]) +
-                                             dot3x<1>(gk[0], oj[0], gk[1], oj[1], gk[2], oj[2]),
-                                         m + sc.word(kVjpT + j) + sc.word(kVjpT + k)));
+        const int64_t x = dot3x<1>(gj[0], ok_[0], gj[1], ok_[1], gj[2], ok_[2]) +
+                          dot3x<1>(gk[0], oj[0], gk[1], oj[1], gk[2], oj[2]);
+        if constexpr (INT) {
+          mx |= mag(x >> 1);
+          sc.put(kVjpX + q, x >> 1);
+        } else {
+          sc.put_real(kVjpX + q, to_double(x, m + sc.word(kVjpT + j) + sc.word(kVjpT + k)));
+        }
       }
     }
     // Tb = b4 (Om^T gp + G^T cw), staub = -s24 cw . gp
@@ -145,6 +165,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
 #pragma unroll
       for (int i = 0; i < 3; ++i)
         m = imax(m, imax(egp + eO[i] + t[i], ecw + eG[i] + t[i]));
+      ea = m;
       Limb a[3], b[3], d[3], f[3];
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
@@ -155,14 +176,36 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
         f[i] = limb(gp);
       }
 #pragma unroll 1
-      for (int j = 0; j < 3; ++j)
-        sc.put_real(kVjpX + 6 + j,
-                    to_double(dot3x<1>(a[0], limb(row(4, j)), a[1], limb(row(5, j)), a[2], limb(row(6, j))) +
-                                  dot3x<1>(b[0], limb(row(0, j)), b[1], limb(row(1, j)), b[2], limb(row(2, j))),
-                              m + sc.word(kVjpT + j) + 1));
-      staub = -s24 * to_double(dot3x<1>(d[0], f[0], d[1], f[1], d[2], f[2]), ecw + egp + 2 * tmax + 1);
+      for (int j = 0; j < 3; ++j) {
+        const int64_t x =
+            dot3x<1>(a[0], limb(row(4, j)), a[1], limb(row(5, j)), a[2], limb(row(6, j))) +
+            dot3x<1>(b[0], limb(row(0, j)), b[1], limb(row(1, j)), b[2], limb(row(2, j)));
+        if constexpr (INT) {
+          ma |= mag(x >> 1);
+          sc.put(kVjpX + 6 + j, x >> 1);
+        } else {
+          sc.put_real(kVjpX + 6 + j, to_double(x, m + sc.word(kVjpT + j) + 1));
+        }
+      }
+      const int64_t x = dot3x<1>(d[0], f[0], d[1], f[1], d[2], f[2]);
+      if constexpr (INT)
+        st = mul8(limb(mul8(inv, nsrhs::fixed::limb(-kTwoThirds61))), limb(x));
+      else
+        staub = -s24 * to_double(x, ecw + egp + 2 * tmax + 1);
     }
-    {
+    if constexpr (INT) {
+      const int nx = norm_shift(mx), na = norm_shift(ma);
+      const Limb a2 = limb(mul8(inv, P.a2.m)), b4 = limb(mul8(inv, P.b4.m));
+      eM = P.a2.e + einv + ex + kap + 4 - nx;
+      eA = P.b4.e + einv + ea + 3 - na;
+#pragma unroll
+      for (int q = 0; q < 6; ++q) Mq[q] = limb(mul8(a2, limb(shl(sc.get(kVjpX + q), nx))));
+#pragma unroll
+      for (int j = 0; j < 3; ++j) A[j] = mul8(b4, limb(shl(sc.get(kVjpX + 6 + j), na)));
+      const int ns = norm_shift(mag(st));
+      eB = einv + ecw + egp + 2 * tmax - 6 - ns;
+      st = shl(st, ns);
+    } else {
       double x[6];
 #pragma unroll
       for (int q = 0; q < 6; ++q) x[q] = sc.real(kVjpX + q);
@@ -199,8 +242,10 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
   const double k2 = P.k2 * rh;
   int ete = 0;
   int64_t tme = 0;
+  if constexpr (!INT) {
 #pragma unroll
-  for (int i = 0; i < 3; ++i) S[i] = (raw(i, 0) + raw(i, 1)) + (raw(i, 2) + raw(i, 3));
+    for (int i = 0; i < 3; ++i) S[i] = (raw(i, 0) + raw(i, 1)) + (raw(i, 2) + raw(i, 3));
+  }
   if constexpr (TAUE) {
     const double sm = fmac(S[2], S[2], fmac(S[1], S[1], S[0] * S[0])) * 0.0625;
     yr_e = M::rsqrt_(sm);
@@ -223,7 +268,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
       const double y = k2a * M::rsqrt_(s);                         // alpha^2 k2 / |u_g|
       const double tau = M::rcp(fmac(y, s, k1));
       sc.put_real(kVjpX + 3 * g, tau);
-      sc.put_real(kVjpX + 3 * g + 1, y * 5.0);  // alpha^2 = 1/5
+      sc.put_real(kVjpX + 3 * g + 1, y);
       stau += tau;
       et = scalar_exp(tau);
     }
@@ -233,15 +278,13 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
       sc.put(kVjpU + 4 * j + g, limb(w[j]));
     }
     const int n = norm_shift(mag(w[0]) | mag(w[1]) | mag(w[2]));
-    sc.put_word(kVjpXg + g, n);
+    sc.put_word(kVjpXg + 3 * g, n);
     theta = imax(theta, et - n);
   }
 
   // ---- T, Q; Qp = a2 Q + a1 I, sT = b4 T ----
   Limb Qp[6], sT[3];
   int eP, eT;
-  int einv;
-  const Limb inv = limb(scalar_fixed(inv_det, einv));
   {
     int64_t Tc[3] = {0, 0, 0}, V[3] = {0, 0, 0};
     Acc q[6];
@@ -254,15 +297,61 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
       int64_t tm = tme;
       if constexpr (!TAUE) tm = scalar_fixed(sc.real(kVjpX + 3 * g), et);
       const Limb tl = limb(tm);
-      const int n = sc.word(kVjpXg + g), k = theta - (et - n);
-      Limb v[3], w[3];
+      const int n = sc.word(kVjpXg + 3 * g), k = theta - (et - n);
+      Limb v[3], w[3], wn[3];
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
         w[j] = sc.limb(kVjpU + 4 * j + g);
-        const int64_t x = whole(w[j]), y = shr(mul8(tl, limb(shl(x, n))), k);
+        const int64_t x = whole(w[j]);
+        wn[j] = limb(shl(x, n));
+        const int64_t y = shr(mul8(tl, wn[j]), k);
         Tc[j] += y;
         v[j] = limb(y);
         V[j] += x;
+      }
+      if constexpr (INT) {
+        // alpha u_g-bar = tau (alpha Tb + 2 N) + alpha^2 sc W, N = alpha^2 Qh W,
+        // alpha^2 sc = (alpha^2 k2 / |u_g|) (-tau^2) (staub + W . (alpha Tb + N))
+        int64_t N[3], Y[3];
+        N[0] = dot3x<3>(Mq[0], wn[0], Mq[3], wn[1], Mq[4], wn[2]);
+        N[1] = dot3x<3>(Mq[3], wn[0], Mq[1], wn[1], Mq[5], wn[2]);
+        N[2] = dot3x<3>(Mq[4], wn[0], Mq[5], wn[1], Mq[2], wn[2]);
+        int eY = imax(eM - n, eA) + 3;
+        const int dN = eY - (eM - n), dA = eY - eA;
+        uint32_t m = 0;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          N[i] = shr(N[i], dN);
+          Y[i] = shr(A[i], dA) + N[i];
+          m |= mag(Y[i]) | mag(N[i]);
+        }
+        const int nY = norm_shift(m) - 1;
+        eY -= nY;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          N[i] = shl(Y[i] + N[i], nY);
+          Y[i] = shl(Y[i], nY);
+        }
+        const int eD = eY + kap - n, eb = imax(eD, eB) + 1;
+        const int64_t tb =
+            shr(dot3x<1>(limb(Y[0]), wn[0], limb(Y[1]), wn[1], limb(Y[2]), wn[2]), eb - eD) +
+            shr(st, eb - eB);
+        const int nb = norm_shift(mag(tb));
+        int ey;
+        const double yd = sc.real(kVjpX + 3 * g + 1);
+        int64_t ym = scalar_fixed(yd, ey);
+        if (yd == 0.0) ym = 0;  // at rest
+        const Limb ty = limb(mul8(limb(mul8(tl, limb(tm * 2))), limb(ym * 2)));
+        const Limb s2 = limb(-mul8(ty, limb(shl(tb, nb))));
+        const int es = 2 * et + ey + eb - nb + 6 + kap - n;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          const int64_t x = mul8(tl, limb(N[i])), y = mul8(s2, wn[i]);
+          const int nx = norm_shift(mag(x)), ny = norm_shift(mag(y));
+          const int ex = et + eY + t[i] - nx, ey = es - t[i] - ny, e = imax(ex, ey) + 1;
+          sc.put(kVjpX + 3 * g + i, shr(shl(x, nx), e - ex) + shr(shl(y, ny), e - ey));
+          sc.put_word(kVjpXg + 3 * g + i, e);
+        }
       }
       mac(q[0], v[0], w[0]);
       mac(q[1], v[1], w[1]);
@@ -290,10 +379,27 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
 #pragma unroll
       for (int j = 0; j < 3; ++j)
         sc.put(kVjpU + 4 * j + a, limb(whole(sc.limb(kVjpU + 4 * j + a)) - V[j]));
+    if constexpr (INT) {
+      // (QA - QB) u_a-bar + QB sum_g u_g-bar, QB = alpha beta
+#pragma unroll 1
+      for (int i = 0; i < 3; ++i) {
+        int e[4];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) e[g] = sc.word(kVjpXg + 3 * g + i);
+        const int m = imax(imax(e[0], e[1]), imax(e[2], e[3])) + 1;
+        int64_t x[4];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) x[g] = shr(sc.get(kVjpX + 3 * g + i), m - e[g]);
+        const int64_t U = beta_sum_wide((x[0] + x[1]) + (x[2] + x[3]));
+#pragma unroll
+        for (int g = 0; g < 4; ++g) sc.put(kVjpX + 3 * g + i, x[g] + U);
+        sc.put_word(kVjpXg + i, m - 4);
+      }
+    }
   }
 
   // ---- FP64: reverse sweep at the Gauss points ----
-  {
+  if constexpr (!INT) {
     double Os[3][3];
     if constexpr (SKEW) {
       const double r48 = P.P.rho * (1.0 / 48.0);
@@ -344,7 +450,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
         const double taub = fmac(ug[2], QT[2], fmac(ug[1], QT[1], fmac(ug[0], QT[0], staub)));
         const double db = -(tau * tau) * taub;
         if constexpr (VREMAN) mub = fmac(crh2, db, mub);
-        const double scl = kyr * db;
+        const double scl = 5.0 * kyr * db;  // alpha^2 = 1/5
 #pragma unroll
         for (int i = 0; i < 3; ++i) ub[i] = fmac(tau, fmac(2.0, QT[i], -Tb[i]), scl * ug[i]);
       } else {
@@ -407,7 +513,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
   for (int i = 0; i < 4; ++i) {
     Limb Kl[3], Hl[3];
     int64_t base;
-    int e;
+    int e, nr = 0;
     if (i < 3) {
       const int eo = sc.word(kVjpEg + 4 + i), ti = sc.word(kVjpT + i), ewi = sc.word(kVjpEu + 4 + i);
       const int e1 = eo + eP, e3 = ecw + ti + eT, e5 = epb + ti, e6 = P.m120.e + ewi + kap + 4;
@@ -416,6 +522,10 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
       const int eh = P.m120.e + ti;
 #pragma unroll
       for (int k = 0; k < 3; ++k) eF = imax(eF, eh + eG[k] + ew[k]);
+      // INT: the Gauss points' part of node a's gradient
+      const int er = INT ? sc.word(kVjpXg + i) : 0;
+      if constexpr (INT) eF = imax(eF, er);
+      uint32_t mh = 0;
       // sum_a w_ai v_a, v_a = m120 (u_a + S)
       Acc wv[3];
 #pragma unroll
@@ -425,6 +535,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
         const Limb wl = limb(sc.get(kVjpW + 4 * i + a));
 #pragma unroll
         for (int j = 0; j < 3; ++j) macx<1>(wv[j], wl, sc.limb(kVjpU + 4 * j + a));
+        if constexpr (INT) mh |= mag(shr(sc.get(kVjpX + 3 * a + i), eF - er));
       }
       Limb Os[3];
       int64_t K[3];
@@ -432,7 +543,6 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
       for (int j = 0; j < 3; ++j) Os[j] = limb(shr(sc.get(kVjpR + 12 + 3 * i + j), eF - e1));
       const Limb cwi = limb(shr(sc.get(kVjpR + 21 + i), eF - e3));
       const int64_t pbi = shr(pb, eF - e5);
-      uint32_t mh = 0;
 #pragma unroll 1
       for (int k = 0; k < 3; ++k) {
         const int64_t h = shr(mul8(P.m120.m, limb(sc.get(kVjpR + 3 * k + i))),
@@ -456,6 +566,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
         Hl[j] = limb(shl(sc.get(kVjpK + j), n));
       }
       base = 0;
+      nr = eF - n - er;
       e = eF - n + 5;
     } else {
       // tr Om / 24 + sum_j c_aj (sum_k sT_k Om_jk - s24 stau cw_j)
@@ -482,9 +593,12 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
       if (i < 3) {
         z = dot3(Hl[0], limb(sc.get(kVjpW + a)), Hl[1], limb(sc.get(kVjpW + 4 + a)), Hl[2],
                  limb(sc.get(kVjpW + 8 + a)), z);
-        x = sc.real(kVjpX + 3 * a + i);
+        if constexpr (INT)
+          z += nr < 0 ? shl(sc.get(kVjpX + 3 * a + i), -nr) : shr(sc.get(kVjpX + 3 * a + i), nr);
+        else
+          x = sc.real(kVjpX + 3 * a + i);
       }
-      out(i, a, to_double(z, e) + x);
+      out(i, a, INT ? to_double(z, e) : to_double(z, e) + x);
     }
   }
   return true;

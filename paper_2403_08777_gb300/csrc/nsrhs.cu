@@ -736,12 +736,12 @@ struct NodalVelocity {
 
 // FP64 adjoint of the elements [e0, e1) (row stride E), one per thread; the
 // two uses, GS and plain as in fwd_fp64_kernel. Integer and FP64 pipe share
-// the sweep (element_fixed_vjp.cuh): FP64 pipe 65 % busy, ALU 41 %. A warp's
-// instructions wait on one another (6.6 clocks each), so the time falls with
-// the warps that share an SM: 12 with 18 KB of scratch a warp, where slots are
-// laid over one another and tau W~ is formed twice rather than kept; 10 with
-// 22 KB took 128^3 7.67 ms, 12 take 7.08 ms. The FP64 form kept the FP64 pipe
-// 90 % busy with 648 instructions: 256^3 114.4 -> 52.2 ms.
+// the sweep (element_fixed_vjp.cuh). A warp's instructions wait on one another
+// (6.6 clocks each), so the time falls with the warps that share an SM: 12
+// with 18 KB of scratch a warp, where slots are laid over one another and
+// tau W~ is formed twice rather than kept; 10 with 22 KB took 128^3 7.67 ms,
+// 12 took 7.08 ms. The FP64 form kept the FP64 pipe 90 % busy with 648
+// instructions: 256^3 114.4 -> 46.3 ms.
 template <int FLAGS, class GS>
 __global__ void __launch_bounds__(kFixedThreads, 12)
     vjp_fp64_kernel(int64_t N, int64_t E, int64_t e0, int64_t e1,
