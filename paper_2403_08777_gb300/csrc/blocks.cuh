@@ -339,16 +339,19 @@ struct NodeSumF32x2 {
 };
 
 // Shared-memory layouts. Staged nodal values: one 4-component record per
-// distinct node (u, v, w, p; the adjoint adds the cotangent's 4), so that an
-// element reads each of its nodes with 128-bit loads. Element entries: one
+// distinct node (u, v, w, p; the adjoint adds one of the cotangent's 4 in an
+// array of its own: interleaved, the records of one kind lie in every second
+// group of banks and the lanes of a load meet twice as often: mixed adjoint at
+// 256^3 4.83 ms, apart 4.56 ms), so that an element reads each of its nodes
+// with 128-bit loads. Element entries: one
 // 4-component record per sorted position.
 template <class R>
 struct Smem;
 template <>
 struct Smem<float> {
-  // the 4 values of node slot lc from a [slot][stride] float buffer
-  static __device__ __forceinline__ void get4(const float* buf, int stride, int lc, float v[4]) {
-    const float4 q = *reinterpret_cast<const float4*>(buf + stride * lc);
+  // the 4 values of node slot lc from a [slot][4] float buffer
+  static __device__ __forceinline__ void get4(const float* buf, int lc, float v[4]) {
+    const float4 q = *reinterpret_cast<const float4*>(buf + 4 * lc);
     v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
   }
   static __device__ __forceinline__ void put4(float* buf, int pos, const float f[4]) {
@@ -374,8 +377,8 @@ struct Smem<float> {
 };
 template <>
 struct Smem<double> {
-  static __device__ __forceinline__ void get4(const double* buf, int stride, int lc, double v[4]) {
-    const double2* q = reinterpret_cast<const double2*>(buf + stride * lc);
+  static __device__ __forceinline__ void get4(const double* buf, int lc, double v[4]) {
+    const double2* q = reinterpret_cast<const double2*>(buf + 4 * lc);
     const double2 a = q[0], b = q[1];
     v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
   }
@@ -524,8 +527,8 @@ __device__ __forceinline__ void block_node_sums2(int64_t N, int nb, const int32_
 // (one block of lead left the staged gathers' latency exposed once the
 // element arithmetic was cheap). A stage holds, for at most `cap` distinct
 // nodes (the mesh's largest block, rounded up to a multiple of 32), the
-// nodal records [cap][W] (W = 4: u, v, w, p; W = 8: and the cotangent), then
-// the node ids [cap] and the runs [cap] of the block. After the stages, the
+// nodal records [cap][4] of u, v, w, p, for W = 8 those of the cotangent
+// likewise, then the node ids [cap] and the runs [cap] of the block. After the stages, the
 // element entries [kBlockSlots][4] by sorted position.
 #ifndef NSRHS_BLOCK_STAGES
 #define NSRHS_BLOCK_STAGES 4
@@ -570,7 +573,7 @@ __device__ __forceinline__ void cp_async_wait() {
 
 // Issues the copies of block b into one pipeline stage: its node ids (stored
 // from the registers that address the gathers), runs, and nodal records
-// (and, for W = 8, the cotangent at columns 4..7).
+// (and, for W = 8, the cotangent's behind them).
 template <class R, int W>
 __device__ __forceinline__ void stage_block(int64_t N, int64_t b,
                                             const int64_t* __restrict__ node_off,
@@ -587,33 +590,34 @@ __device__ __forceinline__ void stage_block(int64_t N, int64_t b,
     const int32_t v = __ldg(nodes + off + j);
     ids[j] = v;
     cp_async<4>(rl + j, runs + off + j);
-    R* slot = vals + W * j;
+    R* slot = vals + 4 * j;
 #pragma unroll
     for (int k = 0; k < 4; ++k) cp_async<sizeof(R)>(slot + k, up + k * N + v);
     if constexpr (W == 8) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) cp_async<sizeof(R)>(slot + 4 + k, cot + k * N + v);
+      for (int k = 0; k < 4; ++k) cp_async<sizeof(R)>(slot + 4 * cap + k, cot + k * N + v);
     }
   }
 }
 
 // The float element routines re-read an element's nodal velocities (and
-// cotangent) from the staged [slot][W] records at their phase boundaries
+// cotangent) from the staged records at their phase boundaries
 // (the empty asm with a memory clobber keeps the compiler from reusing the
 // first loads), so they are not held in registers across the routine: the
 // mixed forward then takes the whole element record one block ahead within
 // its 64 registers, and the mixed adjoint fits 3 CTAs per SM (80 registers)
 // instead of 2 (128).
-template <class R, int W>
+template <class R>
 struct StagedReload {
   const R* vals;
+  int cap;
   const uint32_t* lmv;
   __device__ __forceinline__ void u(R (&uu)[4][3]) const {
     asm volatile("" ::: "memory");
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
       R q[4];
-      Smem<R>::get4(vals, W, (int)(lmv[a] >> 16), q);
+      Smem<R>::get4(vals, (int)(lmv[a] >> 16), q);
       uu[a][0] = q[0];
       uu[a][1] = q[1];
       uu[a][2] = q[2];
@@ -622,7 +626,7 @@ struct StagedReload {
   __device__ __forceinline__ void w(R (&ww)[4][4]) const {
     asm volatile("" ::: "memory");
 #pragma unroll
-    for (int a = 0; a < 4; ++a) Smem<R>::get4(vals + 4, W, (int)(lmv[a] >> 16), ww[a]);
+    for (int a = 0; a < 4; ++a) Smem<R>::get4(vals + 4 * cap, (int)(lmv[a] >> 16), ww[a]);
   }
 };
 
@@ -687,7 +691,7 @@ __global__ void __launch_bounds__(kBlockElems, block_kernel_min_ctas<R>())
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
         R q[4];
-        Smem<R>::get4(vals, 4, (int)(lmv[a] >> 16), q);
+        Smem<R>::get4(vals, (int)(lmv[a] >> 16), q);
         u[a][0] = q[0];
         u[a][1] = q[1];
         u[a][2] = q[2];
@@ -697,7 +701,7 @@ __global__ void __launch_bounds__(kBlockElems, block_kernel_min_ctas<R>())
       cur.geometry(rec, geom64, E, e, c, inv_det, rh);
       R F[4][4];
       if constexpr (sizeof(R) == 4)
-        element_rhs<R, FLAGS>(c, inv_det, rh, u, p, P, F, StagedReload<R, 4>{vals, lmv});
+        element_rhs<R, FLAGS>(c, inv_det, rh, u, p, P, F, StagedReload<R>{vals, cap, lmv});
       else
         element_rhs<R, FLAGS>(c, inv_det, rh, u, p, P, F);
 #pragma unroll
@@ -786,12 +790,12 @@ __device__ __forceinline__ void vjp_block_body(
       for (int a = 0; a < 4; ++a) {
         const int lc = (int)(lmv[a] >> 16);
         R q[4];
-        Smem<R>::get4(vals, 8, lc, q);
+        Smem<R>::get4(vals, lc, q);
         u[a][0] = q[0];
         u[a][1] = q[1];
         u[a][2] = q[2];
         p[a] = q[3];
-        Smem<R>::get4(vals + 4, 8, lc, w[a]);
+        Smem<R>::get4(vals + 4 * cap, lc, w[a]);
       }
       R c[3][3], inv_det, rh;
       cur.geometry(rec, geom64, E, e, c, inv_det, rh);
@@ -800,13 +804,13 @@ __device__ __forceinline__ void vjp_block_body(
         R F[4][4];
         if constexpr (sizeof(R) == 4)
           element_rhs_vjp<R, FLAGS>(c, inv_det, rh, u, p, w, P, F, gu, gp,
-                                    PutRhs<R, StagedReload<R, 8>>{{vals, lmv}, sFr, lmv});
+                                    PutRhs<R, StagedReload<R>>{{vals, cap, lmv}, sFr, lmv});
         else
           element_rhs_vjp<R, FLAGS>(c, inv_det, rh, u, p, w, P, F, gu, gp,
                                     PutRhs<R, NoReload>{{}, sFr, lmv});
       } else {
         if constexpr (sizeof(R) == 4)
-          element_vjp<R, FLAGS>(c, inv_det, rh, u, p, w, P, gu, gp, StagedReload<R, 8>{vals, lmv});
+          element_vjp<R, FLAGS>(c, inv_det, rh, u, p, w, P, gu, gp, StagedReload<R>{vals, cap, lmv});
         else
           element_vjp<R, FLAGS>(c, inv_det, rh, u, p, w, P, gu, gp);
       }
