@@ -285,6 +285,31 @@ __global__ void __launch_bounds__(kBlockElems)
 
 // ---- assembly ----
 
+// Launches of one colour after another. A colour of a small mesh does not fill
+// the chip (64^3: 39300 elements a colour, half of the 2432 resident warps), so
+// its launch takes as long as one element does from gather to scatter, and only
+// the scatters have an order. Each colour's kernel therefore lets the next one
+// start beside it, and waits before its own first add until the one before is
+// complete and its adds are visible (programmatic dependent launch). Without a
+// launch of that kind both calls do nothing. A thread without an element must
+// not wait before the others of its warp have computed theirs: it returns
+// instead, and a launch without any element is left out.
+//   us, one launch after another -> beside one another
+//   FP64 colours (40), forward: 16^3 335 -> 108, 64^3 748 -> 463, 96^3 1911 -> 1525
+//   FP64 colours, adjoint:      16^3 629 -> 198, 64^3 1355 -> 895, 96^3 4456 -> 3889
+//   mixed colours, forward:     16^3 111 -> 60, 64^3 245 -> 214, 96^3 559 -> 554
+//   FP64 block colours, forward: 16^3 412 -> 75, 64^3 1453 -> 1096
+//   mixed block colours, forward: 16^3 50 -> 24, 64^3 120 -> 74
+// The next one starts at the beginning of a kernel (after the gather: 64^3 482
+// us, before the first add: 715); in the mixed colour kernels, which add little
+// arithmetic to the gather, before the first add (at the beginning: 64^3 368 us).
+__device__ __forceinline__ void let_next_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Sum of a node's contributions. double: plain double sum. float: compensated
 // float sum (Knuth's TwoSum keeps the rounding error of every addition), which
 // carries about 48 bits, widened and added in double at the end; this keeps
@@ -659,6 +684,7 @@ __global__ void __launch_bounds__(kBlockElems, block_kernel_min_ctas<R>())
   const int64_t first = COLOUR ? i0 : 0, last = COLOUR ? i1 : n_blocks;
   auto block_at = [&](int64_t i) -> int64_t { return COLOUR ? (int64_t)__ldg(order + i) : i; };
   int64_t i = first + blockIdx.x;
+  if constexpr (COLOUR) let_next_start();
 #pragma unroll 1
   for (int k = 0; k < kStages - 1; ++k) {
     const int64_t ik = i + (int64_t)k * gridDim.x;
@@ -711,6 +737,7 @@ __global__ void __launch_bounds__(kBlockElems, block_kernel_min_ctas<R>())
     const int nb = (int)(__ldg(node_off + b + 1) - __ldg(node_off + b));
     __syncthreads();
     const int32_t* ids = reinterpret_cast<const int32_t*>(st + (size_t)cap * 4 * sizeof(R));
+    if (COLOUR && step == 0) wait_for_previous();
     block_node_sums<R>(N, nb, ids, reinterpret_cast<const uint32_t*>(ids + cap), sF, rhs);
   }
   cp_async_wait<0>();
@@ -757,6 +784,7 @@ __device__ __forceinline__ void vjp_block_body(
   const int64_t first = COLOUR ? i0 : 0, last = COLOUR ? i1 : n_blocks;
   auto block_at = [&](int64_t i) -> int64_t { return COLOUR ? (int64_t)__ldg(order + i) : i; };
   int64_t i = first + blockIdx.x;
+  if constexpr (COLOUR) let_next_start();
 #pragma unroll 1
   for (int k = 0; k < kStages - 1; ++k) {
     const int64_t ik = i + (int64_t)k * gridDim.x;
@@ -825,6 +853,7 @@ __device__ __forceinline__ void vjp_block_body(
     __syncthreads();
     const int32_t* ids = reinterpret_cast<const int32_t*>(st + (size_t)cap * 8 * sizeof(R));
     const uint32_t* rl = reinterpret_cast<const uint32_t*>(ids + cap);
+    if (COLOUR && step == 0) wait_for_previous();
     if constexpr (WITH_F)
       block_node_sums2<R>(N, nb, ids, rl, sFr, rhs, sG, grad);
     else

@@ -527,6 +527,7 @@ __device__ __noinline__ void fwd_fp64_plain(int64_t N, int64_t E, int64_t e,
   gs.get(E, e, v, c, inv_det, rh);
   double F[4][4];
   nsrhs::element_rhs<double, FLAGS>(c, inv_det, rh, u, p, P, F);
+  nsrhs::wait_for_previous();
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -539,16 +540,18 @@ __device__ __forceinline__ int32_t pick(const int32_t v[4], int a) {
 }
 
 // Adds component k of an element's entries to the nodal rows: all four nodes',
-// or that of node a.
+// or that of node a. The first comes with k = 0.
 struct AddEntries {
   double* __restrict__ out;
   int64_t N;
   const int32_t* v;
   __device__ __forceinline__ void operator()(int k, const double f[4]) const {
+    if (k == 0) nsrhs::wait_for_previous();
 #pragma unroll
     for (int a = 0; a < 4; ++a) atomicAdd(out + k * N + v[a], f[a]);
   }
   __device__ __forceinline__ void operator()(int k, int a, double f) const {
+    if (k == 0 && a == 0) nsrhs::wait_for_previous();
     atomicAdd(out + k * N + pick(v, a), f);
   }
 };
@@ -587,6 +590,7 @@ __global__ void __launch_bounds__(kFixedThreads, 16)
   __shared__ int16_t sw[fx::kFwdWords * T];
   const fx::Scratch<T> sc{sq + threadIdx.x, sw + threadIdx.x};
   const int64_t e = e0 + blockIdx.x * (int64_t)T + threadIdx.x;
+  nsrhs::let_next_start();
   if (e >= e1) return;
   if (!plain) {
     int32_t v[4];
@@ -662,6 +666,10 @@ __device__ __forceinline__ void fwd_mixed_element(int64_t N, int64_t E, int64_t 
   nsrhs::load_rec_geometry(rec, e, c, inv_det, rh);
   float F[4][4];
   nsrhs::element_rhs<float, FLAGS>(c, inv_det, rh, u, p, P, F);
+  if constexpr (COLOUR) {
+    nsrhs::let_next_start();
+    nsrhs::wait_for_previous();
+  }
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -715,6 +723,7 @@ __device__ __noinline__ void vjp_fp64_plain(int64_t N, int64_t E, int64_t e,
   gs.get(E, e, v, c, inv_det, rh);
   double gu[4][3], gp[4];
   nsrhs::element_vjp<double, FLAGS>(c, inv_det, rh, u, p, w, P, gu, gp);
+  nsrhs::wait_for_previous();
 #pragma unroll
   for (int a = 0; a < 4; ++a) {
 #pragma unroll
@@ -754,6 +763,7 @@ __global__ void __launch_bounds__(kFixedThreads, 12)
   __shared__ int16_t sw[fx::kVjpWords * T];
   const fx::Scratch<T> sc{sq + threadIdx.x, sw + threadIdx.x};
   const int64_t e = e0 + blockIdx.x * (int64_t)T + threadIdx.x;
+  nsrhs::let_next_start();
   if (e >= e1) return;
   if (!plain) {
     int32_t v[4];
@@ -805,6 +815,10 @@ __device__ __forceinline__ void vjp_mixed_element(int64_t N, int64_t E, int64_t 
   nsrhs::load_rec_geometry(rec, e, c, inv_det, rh);
   float gu[4][3], gp[4];
   nsrhs::element_vjp<float, FLAGS>(c, inv_det, rh, u, p, w, P, gu, gp);
+  if constexpr (COLOUR) {
+    nsrhs::let_next_start();
+    nsrhs::wait_for_previous();
+  }
 #pragma unroll
   for (int a = 0; a < 4; ++a) {
 #pragma unroll
@@ -899,6 +913,24 @@ struct DeviceGuard {
     if (prev >= 0 && cudaGetDevice(&cur) == cudaSuccess && cur != prev) cudaSetDevice(prev);
   }
 };
+
+// Launches a kernel; after: beside the launch before it, for kernels that wait
+// for that one themselves (wait_for_previous).
+template <class... Params, class... Args>
+cudaError_t launch_kernel(void (*kern)(Params...), unsigned grid, unsigned threads, size_t smem,
+                          cudaStream_t s, bool after, Args... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = after ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+}
 
 // Calls f(std::integral_constant<int, FLAGS>) for the runtime formulation flags.
 template <class Fn>
@@ -1470,9 +1502,9 @@ nsrhs_status nsrhs_assemble(const nsrhs_mesh* m, const nsrhs_params* p, const vo
           auto kern = nsrhs::fwd_block_kernel<double, decltype(fl)::value, true>;
           err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
           if (err == cudaSuccess)
-            kern<<<grid, nsrhs::kBlockElems, smem, s>>>(
-                N, E, nb, m->blk_node_off, m->blk_nodes, m->blk_runs, m->blk_cap, m->rec,
-                m->geom, (const double*)up, P, rhs, m->bcol_order, i0, i1);
+            err = launch_kernel(kern, grid, nsrhs::kBlockElems, smem, s, k > 0, N, E, nb,
+                                m->blk_node_off, m->blk_nodes, m->blk_runs, m->blk_cap, m->rec,
+                                m->geom, (const double*)up, P, rhs, m->bcol_order, i0, i1);
         });
       } else {
         auto P = elem_params<float>(p);
@@ -1481,9 +1513,9 @@ nsrhs_status nsrhs_assemble(const nsrhs_mesh* m, const nsrhs_params* p, const vo
           auto kern = nsrhs::fwd_block_kernel<float, decltype(fl)::value, true>;
           err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
           if (err == cudaSuccess)
-            kern<<<grid, nsrhs::kBlockElems, smem, s>>>(
-                N, E, nb, m->blk_node_off, m->blk_nodes, m->blk_runs, m->blk_cap, m->rec,
-                nullptr, (const float*)up, P, rhs, m->bcol_order, i0, i1);
+            err = launch_kernel(kern, grid, nsrhs::kBlockElems, smem, s, k > 0, N, E, nb,
+                                m->blk_node_off, m->blk_nodes, m->blk_runs, m->blk_cap, m->rec,
+                                nullptr, (const float*)up, P, rhs, m->bcol_order, i0, i1);
         });
       }
       if (err == cudaSuccess) err = cudaGetLastError();
@@ -1494,23 +1526,26 @@ nsrhs_status nsrhs_assemble(const nsrhs_mesh* m, const nsrhs_params* p, const vo
     // one launch per colour, in colour order
     for (size_t k = 0; k + 1 < m->col_off.size(); ++k) {
       const int64_t e0 = m->col_off[k], e1 = m->col_off[k + 1];
+      if (e0 == e1) continue;  // a launch waits for the one before only where it has elements
       const unsigned grid = grid_for(e1 - e0, m->device, 16);
+      cudaError_t err = cudaSuccess;
       if (p->precision == NSRHS_FP64) {
         const FixedParams P = fixed_params(p);
         with_flags(flags, [&](auto fl) {
-          fwd_fp64_kernel<decltype(fl)::value, GeomCached>
-              <<<fixed_grid(e1 - e0), kFixedThreads, 0, s>>>(
-                  N, E, e0, e1, m->col_conn, GeomCached{m->col_geom}, (const double*)up, P,
-                  !P.in_range, rhs);
+          err = launch_kernel(fwd_fp64_kernel<decltype(fl)::value, GeomCached>,
+                              fixed_grid(e1 - e0), kFixedThreads, 0, s, k > 0, N, E, e0, e1,
+                              m->col_conn, GeomCached{m->col_geom}, (const double*)up, P,
+                              !P.in_range, rhs);
         });
       } else {
         auto P = elem_params<float>(p);
         with_flags(flags, [&](auto fl) {
-          fwd_mixed_colour_kernel<decltype(fl)::value><<<grid, kThreads, 0, s>>>(
-              N, E, e0, e1, m->col_conn, m->col_rec, (const float*)up, P, rhs);
+          err = launch_kernel(fwd_mixed_colour_kernel<decltype(fl)::value>, grid, kThreads, 0, s,
+                              k > 0, N, E, e0, e1, m->col_conn, m->col_rec, (const float*)up, P,
+                              rhs);
         });
       }
-      NSRHS_TRY(cudaGetLastError());
+      NSRHS_TRY(err);
     }
     return NSRHS_OK;
   }
@@ -1620,9 +1655,9 @@ nsrhs_status nsrhs_assemble_vjp(const nsrhs_mesh* m, const nsrhs_params* p, cons
                         const auto& P) {
         err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (err == cudaSuccess)
-          kern<<<grid, nsrhs::kBlockElems, smem, s>>>(
-              N, E, nb, m->blk_node_off, m->blk_nodes, m->blk_runs, m->blk_cap, m->rec,
-              geom, u, c, P, grad, coloured ? m->bcol_order : nullptr, i0, i1);
+          err = launch_kernel(kern, grid, nsrhs::kBlockElems, smem, s, k > 0, N, E, nb,
+                              m->blk_node_off, m->blk_nodes, m->blk_runs, m->blk_cap, m->rec,
+                              geom, u, c, P, grad, coloured ? m->bcol_order : nullptr, i0, i1);
       };
       if (p->precision == NSRHS_FP64) {
         auto P = elem_params<double>(p);
@@ -1655,24 +1690,26 @@ nsrhs_status nsrhs_assemble_vjp(const nsrhs_mesh* m, const nsrhs_params* p, cons
   if (p->scatter == NSRHS_SCATTER_COLOUR) {
     for (size_t k = 0; k + 1 < m->col_off.size(); ++k) {
       const int64_t e0 = m->col_off[k], e1 = m->col_off[k + 1];
+      if (e0 == e1) continue;  // a launch waits for the one before only where it has elements
       const unsigned grid = grid_for(e1 - e0, m->device, 16);
+      cudaError_t err = cudaSuccess;
       if (p->precision == NSRHS_FP64) {
         const FixedParams P = fixed_params(p);
         with_flags(formulation_flags(p), [&](auto fl) {
-          vjp_fp64_kernel<decltype(fl)::value, GeomCached>
-              <<<fixed_grid(e1 - e0), kFixedThreads, 0, s>>>(
-                  N, E, e0, e1, m->col_conn, GeomCached{m->col_geom}, (const double*)up,
-                  (const double*)cot, P, !P.in_range, grad);
+          err = launch_kernel(vjp_fp64_kernel<decltype(fl)::value, GeomCached>,
+                              fixed_grid(e1 - e0), kFixedThreads, 0, s, k > 0, N, E, e0, e1,
+                              m->col_conn, GeomCached{m->col_geom}, (const double*)up,
+                              (const double*)cot, P, !P.in_range, grad);
         });
       } else {
         auto P = elem_params<float>(p);
         with_flags(formulation_flags(p), [&](auto fl) {
-          vjp_mixed_colour_kernel<decltype(fl)::value><<<grid, kThreads, 0, s>>>(
-              N, E, e0, e1, m->col_conn, m->col_rec, (const float*)up, (const float*)cot, P,
-              grad);
+          err = launch_kernel(vjp_mixed_colour_kernel<decltype(fl)::value>, grid, kThreads, 0, s,
+                              k > 0, N, E, e0, e1, m->col_conn, m->col_rec, (const float*)up,
+                              (const float*)cot, P, grad);
         });
       }
-      NSRHS_TRY(cudaGetLastError());
+      NSRHS_TRY(err);
     }
     return NSRHS_OK;
   }
@@ -1730,9 +1767,9 @@ nsrhs_status nsrhs_assemble_rhs_vjp(const nsrhs_mesh* m, const nsrhs_params* p, 
                         const auto& P) {
         err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (err == cudaSuccess)
-          kern<<<grid, nsrhs::kBlockElems, smem, s>>>(
-              N, E, nb, m->blk_node_off, m->blk_nodes, m->blk_runs, m->blk_cap, m->rec, geom, u,
-              c, P, rhs, grad, coloured ? m->bcol_order : nullptr, i0, i1);
+          err = launch_kernel(kern, grid, nsrhs::kBlockElems, smem, s, k > 0, N, E, nb,
+                              m->blk_node_off, m->blk_nodes, m->blk_runs, m->blk_cap, m->rec, geom,
+                              u, c, P, rhs, grad, coloured ? m->bcol_order : nullptr, i0, i1);
       };
       if (p->precision == NSRHS_FP64) {
         auto P = elem_params<double>(p);
