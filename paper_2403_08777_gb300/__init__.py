@@ -310,8 +310,8 @@ def assemble_host(mesh: Mesh, up_host: torch.Tensor, params: Params | None = Non
 class StepGraph:
     """`steps` explicit time steps of up (in place) captured once in a CUDA
     graph and replayed with one launch: for small meshes, where the steps'
-    kernel launches (each Runge-Kutta stage is a memset, an assembly and an
-    update) cost more than their work. The library calls allocate nothing and
+    kernel launches (each Runge-Kutta stage is an assembly and an update)
+    cost more than their work. The library calls allocate nothing and
     never synchronise, so they can be captured; the graph is bound to the
     addresses of `up` and of its own work buffer.
 

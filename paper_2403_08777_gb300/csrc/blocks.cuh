@@ -309,6 +309,11 @@ __device__ __forceinline__ void let_next_start() {
 __device__ __forceinline__ void wait_for_previous() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// For a kernel that takes its input from the launch before it.
+__device__ __forceinline__ void wait_then_let_next_start() {
+  wait_for_previous();
+  let_next_start();
+}
 
 // Sum of a node's contributions. double: plain double sum. float: compensated
 // float sum (Knuth's TwoSum keeps the rounding error of every addition), which
@@ -675,8 +680,8 @@ __global__ void __launch_bounds__(kBlockElems, block_kernel_min_ctas<R>())
                      const int32_t* __restrict__ nodes, const uint32_t* __restrict__ runs,
                      int cap, const RecChunk* __restrict__ rec, const double* __restrict__ geom64,
                      const R* __restrict__ up, ElemParams<R> P, double* __restrict__ rhs,
-                     const int32_t* __restrict__ order = nullptr, int64_t i0 = 0,
-                     int64_t i1 = 0) {
+                     const int32_t* __restrict__ order, int64_t i0, int64_t i1, bool chain) {
+  if (chain) wait_for_previous();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const size_t sbytes = stage_bytes<R, 4>(cap);
   R* sF = reinterpret_cast<R*>(smem_raw + kStages * sbytes);  // [kBlockSlots][4] entries
@@ -684,7 +689,7 @@ __global__ void __launch_bounds__(kBlockElems, block_kernel_min_ctas<R>())
   const int64_t first = COLOUR ? i0 : 0, last = COLOUR ? i1 : n_blocks;
   auto block_at = [&](int64_t i) -> int64_t { return COLOUR ? (int64_t)__ldg(order + i) : i; };
   int64_t i = first + blockIdx.x;
-  if constexpr (COLOUR) let_next_start();
+  let_next_start();
 #pragma unroll 1
   for (int k = 0; k < kStages - 1; ++k) {
     const int64_t ik = i + (int64_t)k * gridDim.x;
@@ -737,7 +742,7 @@ __global__ void __launch_bounds__(kBlockElems, block_kernel_min_ctas<R>())
     const int nb = (int)(__ldg(node_off + b + 1) - __ldg(node_off + b));
     __syncthreads();
     const int32_t* ids = reinterpret_cast<const int32_t*>(st + (size_t)cap * 4 * sizeof(R));
-    if (COLOUR && step == 0) wait_for_previous();
+    if (step == 0) wait_for_previous();
     block_node_sums<R>(N, nb, ids, reinterpret_cast<const uint32_t*>(ids + cap), sF, rhs);
   }
   cp_async_wait<0>();
@@ -784,7 +789,7 @@ __device__ __forceinline__ void vjp_block_body(
   const int64_t first = COLOUR ? i0 : 0, last = COLOUR ? i1 : n_blocks;
   auto block_at = [&](int64_t i) -> int64_t { return COLOUR ? (int64_t)__ldg(order + i) : i; };
   int64_t i = first + blockIdx.x;
-  if constexpr (COLOUR) let_next_start();
+  let_next_start();
 #pragma unroll 1
   for (int k = 0; k < kStages - 1; ++k) {
     const int64_t ik = i + (int64_t)k * gridDim.x;
@@ -853,7 +858,7 @@ __device__ __forceinline__ void vjp_block_body(
     __syncthreads();
     const int32_t* ids = reinterpret_cast<const int32_t*>(st + (size_t)cap * 8 * sizeof(R));
     const uint32_t* rl = reinterpret_cast<const uint32_t*>(ids + cap);
-    if (COLOUR && step == 0) wait_for_previous();
+    if (step == 0) wait_for_previous();
     if constexpr (WITH_F)
       block_node_sums2<R>(N, nb, ids, rl, sFr, rhs, sG, grad);
     else
