@@ -14,7 +14,7 @@ pressure ~ U(-1, 1), seeded and synthetic.
 
 Prints one JSON line (rank 0): `value` from the device-resident step,
 `e2e` through StepPipeline from pinned host buffers, `roofline` for the
-dominant kernel (the adjoint) against the FP64 pipe rate, `cpu_baseline`
+dominant kernel (the adjoint) against the issue rate, `cpu_baseline`
 (the oracle on the host cores), sampled clocks, and under `forms` the other
 configurations: formulation variants, the one-pass RHS + adjoint, the
 element-matrix comparison path, explicit SSP-RK3 steps (and small-mesh steps
@@ -72,8 +72,8 @@ FLOPS_GEOMETRY = 43
 # ncu capture of each kernel on the 128^3-hex RCM mesh, scaled to a launch by
 # the element count (traffic grows in proportion). None once a kernel has
 # changed since its counters were taken.
-DRAM_BYTES_PER_TET = {"fwd_fp64": 157.7, "vjp_fp64": 187.9,
-                      "fwd_mixed": 92.4, "vjp_mixed": 106.6}
+DRAM_BYTES_PER_TET = {"fwd_fp64": 127.5, "vjp_fp64": 137.5,
+                      "fwd_mixed": 92.5, "vjp_mixed": 107.6}
 
 # Algorithmic (compulsory) bytes per tet with ideal node reuse (N/E = 0.1686
 # on the Kuhn mesh): connectivity or block map 16, cached geometry 88 (f64) or
@@ -83,6 +83,13 @@ ALG_BYTES_PER_TET = {"fwd_fp64": 120.0, "vjp_fp64": 126.0, "fwd_mixed": 75.0, "v
 
 # FP64 FMA lanes per SM per clock on GB300 (1.25 TF/s nominal at 2.07 GHz).
 FP64_LANES_PER_SM = 2
+
+# Warp instructions per 32 tets (smsp__inst_executed.sum of the same captures):
+# the FP64 kernels do most of the element in block fixed-point arithmetic on the
+# integer pipe, so their roof is the issue rate of the four schedulers of an SM,
+# not the FP64 pipe, which they pass (frac_fp64_pipe above 1).
+WARP_INSTR_PER_32_TETS = {"fwd_fp64": 4827, "vjp_fp64": 9699}
+WARP_INSTR_PER_SM_PER_CLOCK = 4
 
 
 def parse():
@@ -464,7 +471,7 @@ def run_ours(args):
     # FP64 pipe peak from the hardware rate: 2 FP64 FMA lanes per SM per clock
     # (GB300's nominal 1.25 TF/s at 2.07 GHz on 152 SMs), at the SM clock
     # sampled during the timed region. The FMA-chain probe reaches ~84 % of
-    # the pipe (ncu), the element kernels ~89 %, so the probe under-states it.
+    # the pipe (ncu).
     n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
     clk_mhz = clocks.get("sm_mhz") or 2070.0
     fp64_peak = FP64_LANES_PER_SM * 2 * n_sm * clk_mhz * 1e6 / 1e12
@@ -635,26 +642,32 @@ def run_ours(args):
         except Exception as exc:  # an auxiliary form must not cost the bench line
             forms["partitioned_one_gpu"] = {"error": repr(exc)}
 
+    # the FP64 kernels against the issue rate
+    issue_peak = WARP_INSTR_PER_SM_PER_CLOCK * n_sm * clk_mhz * 1e6 / 1e9
+
+    def issue_roofline(key, ms):
+        ach = WARP_INSTR_PER_32_TETS[key] * w.n_elems / 32 / (ms * 1e-3) / 1e9
+        return {"bound": "alu", "kernel": key, "achieved": ach, "peak": issue_peak,
+                "unit": "G warp instructions/s", "frac": ach / issue_peak,
+                "peak_source": f"issue rate: {WARP_INSTR_PER_SM_PER_CLOCK} warp instructions per "
+                               f"SM and clock x {n_sm} SMs x {clk_mhz:.0f} MHz sampled during "
+                               f"the timed region",
+                "warp_instr_per_32_tets": WARP_INSTR_PER_32_TETS[key],
+                "tflops_algorithmic": forms[key]["tflops"],
+                "frac_fp64_pipe": forms[key]["frac_fp64_pipe"], "launch_ms": ms}
+
     dom = "vjp_fp64" if vjp_med >= fwd_med else "fwd_fp64"
     dom_ms = vjp_med if dom == "vjp_fp64" else fwd_med
-    achieved = forms[dom]["tflops"]
-    roofline = {"bound": "alu", "kernel": dom, "achieved": achieved, "peak": fp64_peak,
-                "unit": "TFLOP/s", "frac": achieved / fp64_peak,
-                "traffic": (DRAM_BYTES_PER_TET[dom] * w.n_elems
-                            if DRAM_BYTES_PER_TET.get(dom) is not None else None),
-                "peak_source": (f"FP64 pipe rate: {FP64_LANES_PER_SM} FMA lanes/SM/clock x 2 flops "
-                                f"x {n_sm} SMs x {clk_mhz:.0f} MHz sampled during the timed "
-                                f"region (FP64 is not in MEASURED_PEAKS.json); the FMA-chain "
-                                f"probe measured {fp64_probe:.3f} TF/s in this run"),
-                "flops_per_tet": flops["vjp" if dom == "vjp_fp64" else "fwd"],
-                "launch_ms": dom_ms}
+    roofline = issue_roofline(dom, dom_ms)
+    roofline["traffic"] = (DRAM_BYTES_PER_TET[dom] * w.n_elems
+                           if DRAM_BYTES_PER_TET.get(dom) is not None else None)
+    roofline["flops_per_tet"] = flops["vjp" if dom == "vjp_fp64" else "fwd"]
     # the same launch counted with the method's own operations (the oracle's
     # definition): what the restructured algebra does in fewer operations
     mflops = FLOPS_PER_TET_METHOD_VREMAN if w.c_vreman else FLOPS_PER_TET_METHOD
     mper = mflops["vjp" if dom == "vjp_fp64" else "fwd"]
     roofline["flops_per_tet_method"] = mper
-    roofline["achieved_method"] = mper * w.n_elems / (dom_ms * 1e-3) / 1e12
-    roofline["frac_method"] = roofline["achieved_method"] / fp64_peak
+    roofline["tflops_method"] = mper * w.n_elems / (dom_ms * 1e-3) / 1e12
     # the mixed-precision kernels against both of their roofs: FP32 FMA (the
     # live probe) and HBM (algorithmic bytes against the measured copy peak)
     roofline_mixed = {}
@@ -668,12 +681,9 @@ def run_ours(args):
             "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": bench_config(w, world),
             "roofline": roofline,
-            "roofline_fwd": {"bound": "alu", "achieved": forms["fwd_fp64"]["tflops"],
-                             "peak": fp64_peak, "unit": "TFLOP/s",
-                             "frac": forms["fwd_fp64"]["tflops"] / fp64_peak,
-                             "flops_per_tet": flops["fwd"],
+            "roofline_fwd": {**issue_roofline("fwd_fp64", fwd_med), "flops_per_tet": flops["fwd"],
                              "flops_per_tet_method": mflops["fwd"],
-                             "achieved_method": mflops["fwd"] * w.n_elems / (fwd_med * 1e-3) / 1e12},
+                             "tflops_method": mflops["fwd"] * w.n_elems / (fwd_med * 1e-3) / 1e12},
             "roofline_mixed": roofline_mixed,
             "peaks": {"fp64_tflops": fp64_peak, "fp64_probe_tflops": fp64_probe,
                       "fp32_probe_tflops": fp32_probe,
@@ -700,10 +710,10 @@ MIXED_KERNELS = {"fwd_mixed": "fwd_block_kernel<float,0>", "vjp_mixed": "vjp_blo
 # What ncu shows stopping them (128^3 captures of the current kernels).
 MIXED_LIMITER = {
     "fwd_mixed": "issue latency between barrier phases at 4 CTAs/SM (64 registers): "
-                 "issue 67 %, L1/TEX 78 % (half of the shared wavefronts bank conflicts), "
+                 "issue 67 %, L1/TEX 75 % (half of the shared wavefronts bank conflicts), "
                  "FMA 44 %, DRAM 40 %; top stalls barrier, long scoreboard",
-    "vjp_mixed": "latency at 3 CTAs/SM (80 registers): issue 59 %, warps active 34 %, "
-                 "L1/TEX 71 %, FMA 43 %, DRAM 28 %; top stalls long scoreboard, barrier"}
+    "vjp_mixed": "latency at 3 CTAs/SM (80 registers): issue 61 %, warps active 34 %, "
+                 "L1/TEX 63 %, FMA 44 %, DRAM 29 %; top stalls long scoreboard, barrier"}
 
 
 def mixed_roofline(key, ms, n_elems, fp32_peak, hbm_peak):

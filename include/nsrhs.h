@@ -219,7 +219,8 @@ nsrhs_status nsrhs_assemble_vjp(const nsrhs_mesh* m, const nsrhs_params* p, cons
  * Both of the above at the same state in one pass: rhs = assembled RHS of up
  * and grad = (d rhs / d up)^T cot, with one gather of up and cot per element
  * and the element's forward intermediates computed once (the adjoint's
- * recomputation of them is shared with the RHS). For callers that hold the
+ * recomputation of them is shared with the RHS); NSRHS_FP64 with atomics runs
+ * the forward and the adjoint one after the other, which is faster. For callers that hold the
  * cotangent before the RHS is needed: residual and adjoint-residual sweeps
  * of steady adjoint solvers, one-shot optimisation, Newton-Krylov with a
  * transposed product. Types and layouts as nsrhs_assemble / _vjp; rhs and

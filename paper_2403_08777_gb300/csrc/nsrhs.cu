@@ -5,10 +5,12 @@
 // validation, aspect-ratio classification, Morton element order, cached
 // geometry, element blocks, optional colourings), argument checking and
 // kernel launches. Device side: the element kernels (element.cuh holds the
-// per-element arithmetic, blocks.cuh the block-staged kernels, colour.cuh
-// the colourings). One thread assembles one element, with every
-// intermediate in registers (the paper's specialisation + privatisation,
-// Sec. V-B/V-C), and scatters its 16 entries as soon as they are computed
+// per-element arithmetic, element_fixed.cuh and element_fixed_vjp.cuh its FP64
+// form in block fixed-point numbers, blocks.cuh the block-staged kernels,
+// colour.cuh the colourings). One thread assembles one element, with every
+// intermediate on chip (the paper's specialisation + privatisation,
+// Sec. V-B/V-C: registers, for the FP64 form also the thread's slots in shared
+// memory), and scatters its 16 entries as soon as they are computed
 // (immediate scatter, Sec. V-D): by double-precision atomic adds (the FP64
 // default), by per-block sums staged in shared memory (the mixed default),
 // or in coloured launches, whose atomics never meet at one address, so that
@@ -878,7 +880,7 @@ __global__ void __launch_bounds__(kThreads)
 // (element_rhs_vjp): one gather of (u, p) and the cotangent, one geometry
 // read, the forward intermediates computed once; float arithmetic, double
 // accumulation by integer widening. (The FP64 form runs its forward and its
-// adjoint kernel one after the other: fixed-point forward and adjoint, 23 + 60
+// adjoint kernel one after the other: fixed-point forward and adjoint, 20.5 + 46.3
 // ms at 256^3, against 141 ms for one FP64 pass.)
 template <int FLAGS>
 __global__ void __launch_bounds__(kThreads)
@@ -1586,8 +1588,8 @@ nsrhs_status assemble(const nsrhs_mesh* m, const nsrhs_params* p, const void* up
     }
     return NSRHS_OK;
   }
-  // AUTO: atomics for the FP64 form (its FP64 pipe, not the scatter, is the
-  // limit, and the block sums would add FP64 work); blocks for the mixed form
+  // AUTO: atomics for the FP64 form (its arithmetic, not the scatter, is the
+  // limit, and the block kernels do theirs on the FP64 pipe); blocks for the mixed form
   // (bound by L2 atomics and gathers).
   const bool block = p->scatter == NSRHS_SCATTER_BLOCK ||
                      (p->scatter == NSRHS_SCATTER_AUTO && p->precision == NSRHS_MIXED);
@@ -1687,7 +1689,7 @@ nsrhs_status nsrhs_assemble_vjp(const nsrhs_mesh* m, const nsrhs_params* p, cons
     });
     return cuda_status(err);
   }
-  // AUTO: atomics for the FP64 form (FP64-pipe-bound), blocks for the mixed
+  // AUTO: atomics for the FP64 form (arithmetic-bound), blocks for the mixed
   // form (measured faster)
   const bool block = p->scatter == NSRHS_SCATTER_BLOCK ||
                      (p->scatter == NSRHS_SCATTER_AUTO && p->precision == NSRHS_MIXED);
