@@ -493,7 +493,11 @@ __device__ __forceinline__ void load_geometry(const R* __restrict__ geom, int64_
 // call itself (Sec. V-B's per-element constant gradients, 43 FP64 operations).
 // get(): into registers; stage(): the cofactors into the scratch slots from
 // `at` on, 1/detJ and detJ^(-1/3) into registers.
+// kCopied: stage() only issues copies, before the gather of (u, p); what computes
+// comes behind the gather and hides its latency (64^3 forward with the geometry
+// formed in the call: 386 us before it, 376 behind it).
 struct GeomCached {
+  static constexpr bool kCopied = true;
   const double* __restrict__ geom;
   __device__ __forceinline__ void get(int64_t E, int64_t e, const int32_t v[4], double c[3][3],
                                       double& inv_det, double& rh) const {
@@ -510,6 +514,7 @@ struct GeomCached {
   }
 };
 struct GeomRecompute {
+  static constexpr bool kCopied = false;
   const double* __restrict__ coords;  // [3][N]
   int64_t N;
   __device__ __forceinline__ void get(int64_t E, int64_t e, const int32_t v[4], double c[3][3],
@@ -624,13 +629,14 @@ __global__ void __launch_bounds__(kFixedThreads, 16)
 #pragma unroll
     for (int a = 0; a < 4; ++a) v[a] = ldg(conn + a * E + e);
     double inv_det, rh;
-    gs.stage(sc, fx::kSlotC, E, e, v, inv_det, rh);
+    if constexpr (GS::kCopied) gs.stage(sc, fx::kSlotC, E, e, v, inv_det, rh);
     if (chain) nsrhs::wait_then_let_next_start();
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         nsrhs::cp_async<8>(sc.q + (fx::kSlotU + 4 * i + a) * T, up + i * N + v[a]);
+    if constexpr (!GS::kCopied) gs.stage(sc, fx::kSlotC, E, e, v, inv_det, rh);
     nsrhs::cp_async_commit();
     nsrhs::cp_async_wait<0>();
     if (fx::element_rhs_fixed<FLAGS, T>(sc, inv_det, rh, P, AddEntries{rhs, N, v})) return;
