@@ -386,7 +386,9 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
         int e[4];
 #pragma unroll
         for (int g = 0; g < 4; ++g) e[g] = sc.word(kVjpXg + 3 * g + i);
-        const int m = imax(imax(e[0], e[1]), imax(e[2], e[3])) + 1;
+        // |x| < 2^59, so that |x + U| <= (1 + 4 beta) 2^59 < 2^60.2: every reader
+        // of these slots takes numbers below 2^61
+        const int m = imax(imax(e[0], e[1]), imax(e[2], e[3])) + 2;
         int64_t x[4];
 #pragma unroll
         for (int g = 0; g < 4; ++g) x[g] = shr(sc.get(kVjpX + 3 * g + i), m - e[g]);

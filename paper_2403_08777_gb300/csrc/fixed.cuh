@@ -35,6 +35,12 @@ namespace fixed {
 
 // ---- bits of doubles, and the integer instructions used ----
 
+// What the arithmetic relies on: shift counts that are not negative, no bits lost
+// at the top. A host build that defines it (tests/fixedpoint) counts violations.
+#if !defined(NSRHS_FIXED_EXPECT)
+#define NSRHS_FIXED_EXPECT(ok)
+#endif
+
 #if defined(__CUDA_ARCH__)
 __device__ __forceinline__ int32_t hi_word(double x) { return __double2hiint(x); }
 __device__ __forceinline__ uint32_t lo_word(double x) { return (uint32_t)__double2loint(x); }
@@ -70,10 +76,27 @@ inline uint32_t lo_word(double x) { return (uint32_t)bits_of(x); }
 inline double make_double(uint64_t b) { double x; std::memcpy(&x, &b, 8); return x; }
 inline int clz32(uint32_t x) { return x ? __builtin_clz(x) : 32; }
 inline int imax(int a, int b) { return a > b ? a : b; }
-inline int64_t mad_wide(int32_t a, int32_t b, int64_t c) { return (int64_t)a * b + c; }
-inline int64_t shr(int64_t x, int k) { return x >> (k < 63 ? k : 63); }
-inline uint64_t shru(uint64_t x, int k) { return k > 63 ? 0 : x >> k; }
-inline int64_t shl(int64_t x, int k) { return k > 63 ? 0 : (int64_t)((uint64_t)x << k); }
+inline int64_t mad_wide(int32_t a, int32_t b, int64_t c) {
+  int64_t d;
+  const bool over = __builtin_add_overflow((int64_t)a * b, c, &d);
+  NSRHS_FIXED_EXPECT(!over);
+  (void)over;
+  return d;
+}
+// A negative count is a large one, as for the instructions.
+inline int64_t shr(int64_t x, int k) {
+  NSRHS_FIXED_EXPECT(k >= 0);
+  return x >> ((uint32_t)k < 63u ? k : 63);
+}
+inline uint64_t shru(uint64_t x, int k) {
+  NSRHS_FIXED_EXPECT(k >= 0);
+  return (uint32_t)k > 63u ? 0 : x >> k;
+}
+inline int64_t shl(int64_t x, int k) {
+  const int64_t r = (uint32_t)k > 63u ? 0 : (int64_t)((uint64_t)x << k);
+  NSRHS_FIXED_EXPECT(k >= 0 && shr(r, k) == x);
+  return r;
+}
 #endif
 __device__ __forceinline__ int32_t hi32(int64_t x) { return (int32_t)(x >> 32); }
 
@@ -130,6 +153,7 @@ __device__ __forceinline__ double to_double(int64_t x, int e) {
     k -= 31;
   }
   const int n = clz32(ah);  // n >= 1 (32 for x = 1, where v is still right)
+  NSRHS_FIXED_EXPECT(x == 0 || (k - n >= 0 && k - n < 2046));
   // leading bit to 2^62, then the 53 leading bits rounded
   const uint64_t v = ((uint64_t)shl((int64_t)((uint64_t)ah << 32 | al), n - 1) + 512u) >> 10;
   const uint32_t hi = (uint32_t)(v >> 32) + ((uint32_t)(k - n) << 20);
@@ -145,6 +169,7 @@ struct Limb {
 __device__ __forceinline__ constexpr Limb limb(int64_t x) {
   return {(int32_t)((uint32_t)(x >> 32) + ((uint32_t)x >> 31)), (int32_t)(uint32_t)x};
 }
+__device__ __forceinline__ int64_t top(const Limb& a) { return a.h < 0 ? -(int64_t)a.h : a.h; }
 __device__ __forceinline__ int64_t whole(const Limb& a) {
   return (int64_t)((uint64_t)(uint32_t)(a.h - (int32_t)((uint32_t)a.l >> 31)) << 32 | (uint32_t)a.l);
 }
@@ -169,6 +194,7 @@ __device__ __forceinline__ int64_t mul(const Limb& a, const Limb& b) {
 // is split over both high limbs: a.h may be 2^28 and b.h 2^29 (a mantissa of
 // ones rounds up to the next power of two).
 __device__ __forceinline__ int64_t mul8(const Limb& a, const Limb& b) {
+  NSRHS_FIXED_EXPECT(top(a) <= 1 << 28 && top(b) <= 1 << 29);
   int64_t M = mad_wide(a.h, b.l, 1ll << 31);
   M = mad_wide(a.l, b.h, M);
   return mad_wide(hi32(M), 8, mad_wide(a.h * 4, b.h * 2, 0));
@@ -189,6 +215,7 @@ template <int S>
 __device__ __forceinline__ Acc accx_start(int64_t h = 0) { return {h, 1ll << (31 - S)}; }
 template <int S>
 __device__ __forceinline__ void macx(Acc& s, const Limb& a, const Limb& b) {
+  NSRHS_FIXED_EXPECT(top(a) < 1 << (S == 1 ? 30 : 29) && top(b) < 1ll << (S == 3 ? 30 : 31));
   s.H = mad_wide(a.h * (S == 1 ? 2 : 4), b.h * (S == 3 ? 2 : 1), s.H);
   s.M = mad_wide(a.h, b.l, s.M);
   s.M = mad_wide(a.l, b.h, s.M);

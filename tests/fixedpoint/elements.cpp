@@ -1,0 +1,160 @@
+// Host check of the fixed-point element routines over elements of many kinds,
+// beside check.cpp, whose reference and helpers it uses: what the arithmetic
+// relies on (NSRHS_FIXED_EXPECT: shift counts that are not negative, no bits
+// lost at the top of a number, accumulators and results in range) holds in
+// every element, and the results are those of the double-precision routines.
+// Prints one line per check: "name value limit".
+static long g_violations = 0;
+#define NSRHS_FIXED_EXPECT(ok) (void)((ok) || ++g_violations)
+#define main check_main
+#include "check.cpp"
+#undef main
+
+struct Results {
+  double rhs[4][4], vjp[4][4];  // [node][component]
+};
+template <int FLAGS>
+static bool by_fixed(const Element& q, Results& r) {
+  const auto FP = fixed::make_fixed_params(q.P, (FLAGS & kSkew) != 0);
+  int64_t slots[128];
+  int16_t words[64];
+  stage(q, slots);
+  if (!fixed::element_rhs_fixed<FLAGS, 1>({slots, words}, q.inv, q.rh, FP, Keep{r.rhs})) return false;
+  for (int k = 0; k < 9; ++k) std::memcpy(slots + fixed::kVjpC + k, &q.c[k / 3][k % 3], 8);
+  for (int a = 0; a < 4; ++a) {
+    for (int i = 0; i < 3; ++i) std::memcpy(slots + fixed::kVjpU + 4 * i + a, &q.u[a][i], 8);
+    std::memcpy(slots + fixed::kVjpP + a, &q.p[a], 8);
+    for (int i = 0; i < 4; ++i) std::memcpy(slots + fixed::kVjpW + 4 * i + a, &q.w[a][i], 8);
+  }
+  return fixed::element_vjp_fixed<FLAGS, 1>({slots, words}, q.inv, q.rh, FP,
+                                            [&](int i, int a) { return q.u[a][i]; }, Keep{r.vjp});
+}
+template <int FLAGS>
+static void by_double(const Element& q, Results& r) {
+  double gu[4][3], gp[4];
+  element_rhs<double, FLAGS>(q.c, q.inv, q.rh, q.u, q.p, q.P, r.rhs);
+  element_vjp<double, FLAGS>(q.c, q.inv, q.rh, q.u, q.p, q.w, q.P, gu, gp);
+  for (int a = 0; a < 4; ++a) {
+    for (int i = 0; i < 3; ++i) r.vjp[a][i] = gu[a][i];
+    r.vjp[a][3] = gp[a];
+  }
+}
+
+// Differences of two routines over many elements, norm-wise per component.
+struct Sum {
+  double d[8] = {}, n[8] = {};
+  void add(const Results& x, const Results& ref) {
+    for (int a = 0; a < 4; ++a)
+      for (int k = 0; k < 4; ++k) {
+        d[k] += std::pow(x.rhs[a][k] - ref.rhs[a][k], 2);
+        n[k] += std::pow(ref.rhs[a][k], 2);
+        d[4 + k] += std::pow(x.vjp[a][k] - ref.vjp[a][k], 2);
+        n[4 + k] += std::pow(ref.vjp[a][k], 2);
+      }
+  }
+  double worst() const {
+    double w = 0;
+    for (int k = 0; k < 8; ++k)
+      if (n[k] > 0) w = std::max(w, std::sqrt(d[k] / n[k]));
+    return w;
+  }
+};
+
+// Low velocities: 0 nearly uniform, 1 at one node only (beside a no-slip
+// wall), at the given cell Reynolds number, pressures of order 1.
+static Element low_velocity(int kind, double reynolds, double mu, double flat) {
+  Element q = make(0, 0);
+  for (int a = 0; a < 4; ++a) q.X[a][2] /= flat;
+  element_geometry<double, double>(q.X, q.c, q.inv, q.rh);
+  const double U = reynolds * mu * 64, spread = std::pow(10.0, uni(-8, -1));
+  const double dir[3] = {normal(), normal(), normal()};
+  const int node = (int)(rng() % 4);
+  for (int a = 0; a < 4; ++a)
+    for (int i = 0; i < 3; ++i)
+      q.u[a][i] = kind == 0 ? U * (dir[i] + spread * normal()) : a == node ? U * normal() : 0.0;
+  q.P.mu = mu;
+  return q;
+}
+// The library's tolerance for FP64 results, 1e-12 norm-wise.
+template <int FLAGS>
+static void low_velocities(int n) {
+  for (const int kind : {0, 1})
+    for (const double mu : {1e-4, 1e-2})
+      for (const double flat : {1.0, 20.0}) {
+        Sum s;
+        int left = 0;
+        g_violations = 0;
+        for (int it = 0; it < n; ++it) {
+          const Element q = low_velocity(kind, std::pow(10.0, uni(-2, 0.3)), mu, flat);
+          Results x, ref;
+          by_double<FLAGS>(q, ref);
+          if (!by_fixed<FLAGS>(q, x)) ++left;
+          else s.add(x, ref);
+        }
+        const int id = 100 * kind + 10 * (mu > 1e-3) + (flat > 1);
+        say("low_velocity_expect", FLAGS, id, (double)g_violations, 0);
+        say("low_velocity_left", FLAGS, id, left, 0);
+        // the gradient of a velocity at one node has rank 1, where the eddy
+        // viscosity is the square root of a rounding error in any arithmetic
+        if (kind == 0 || !(FLAGS & kVreman)) say("low_velocity", FLAGS, id, s.worst(), 1e-12);
+      }
+}
+
+// What the arithmetic relies on, for check.cpp's kinds of elements.
+template <int FLAGS>
+static void expectations(int n) {
+  for (int kind = 0; kind < 6; ++kind) {
+    g_violations = 0;
+    for (int it = 0; it < n; ++it) {
+      Results x;
+      by_fixed<FLAGS>(make(kind, it), x);
+    }
+    say("expect", FLAGS, kind, (double)g_violations, 0);
+  }
+}
+
+// A wall cell whose four Gauss points add up alike: their sum needs the last
+// bit that a stored number has.
+static void wall_cell() {
+  Element q = {
+      {{0.73412880520138168, 0.45151404638763065, 0.5609918590211681},
+       {0.74820741898590692, 0.45335968290017303, 0.5620100571258726},
+       {0.75128004838359452, 0.46875315366672304, 0.56210945379511901},
+       {0.75012502088914668, 0.47061793926641393, 0.5794197255459923}},
+      {{0, 0, 0}, {0, 0, 0}, {-0.00029927059211173082, 0.00026118075869641392, 0.00035132161602936465},
+       {0, 0, 0}},
+      {0.93163480449927949, 0.36924891566208573, 0.28743947818824322, -0.78753450712075257},
+      {{-0.22862203235631162, 0.05894589575145668, 0.11511810767374644, -0.65256280448438919},
+       {-0.4568503872610965, -1.33495587783708, -1.2568222182711835, -0.57268009514914131},
+       {1.7422392085597567, -0.56418157997698914, 0.21377690233090399, -0.89421883752649656},
+       {-0.058263528637499638, 1.452970897956954, -1.2989615540193649, -0.98318531139972232}},
+      {}, 0, 0, {1.0, 1e-4, 0.0, 4, 2}};
+  element_geometry<double, double>(q.X, q.c, q.inv, q.rh);
+  Results x, ref;
+  g_violations = 0;
+  by_double<0>(q, ref);
+  say("wall_cell_left", 0, 0, by_fixed<0>(q, x) ? 0 : 1, 0);
+  say("wall_cell_expect", 0, 0, (double)g_violations, 0);
+  Sum s;
+  s.add(x, ref);
+  say("wall_cell", 0, 0, s.worst(), 1e-12);
+}
+
+template <int FLAGS>
+static void all(int n) {
+  expectations<FLAGS>(n / 10);
+  low_velocities<FLAGS>(n);
+}
+
+int main() {
+  wall_cell();
+  all<0>(100000);
+  all<1>(20000);
+  all<2>(20000);
+  all<3>(20000);
+  all<4>(20000);
+  all<5>(20000);
+  all<6>(20000);
+  all<7>(20000);
+  return 0;
+}
