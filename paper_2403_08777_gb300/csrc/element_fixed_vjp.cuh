@@ -20,8 +20,8 @@ namespace nsrhs {
 namespace fixed {
 
 // Slots of element_vjp_fixed, laid over one another so that 12 warps share
-// an SM. U: velocities, component i of node a at kVjpU + 4 i + a; then W, W~
-// and back to u. X: cofactors (input c_k,j at kVjpC + 3 (k - 1) + j, then
+// an SM. U: velocities, component i of node a at kVjpU + 4 i + a; then W
+// and u, aligned. X: cofactors (input c_k,j at kVjpC + 3 (k - 1) + j, then
 // limbs); then the contractions for the Gauss points, tau and k2/|u_g|, and the
 // Gauss points' gradients. W: the cotangent, component i of node a at kVjpW +
 // 4 i + a; the slots of its component 3 end as a row's four sums. R: gradient
@@ -254,7 +254,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
     tme = scalar_fixed(tau_e, ete);
   }
 
-  // ---- per Gauss point: tau_g and k2 / |u_g|, W~, tau W~ ----
+  // ---- per Gauss point: tau_g and k2 / |u_g|, the normalisation of W~ ----
   const double k2a = P.k2a * rh;
   int theta = -32768;
 #pragma unroll 1
@@ -273,10 +273,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
       et = scalar_exp(tau);
     }
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      w[j] = shr(w[j], kap - (eu[j] + t[j]));
-      sc.put(kVjpU + 4 * j + g, limb(w[j]));
-    }
+    for (int j = 0; j < 3; ++j) w[j] = shr(w[j], kap - (eu[j] + t[j]));
     const int n = norm_shift(mag(w[0]) | mag(w[1]) | mag(w[2]));
     sc.put_word(kVjpXg + 3 * g, n);
     theta = imax(theta, et - n);
@@ -301,14 +298,20 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
       Limb v[3], w[3], wn[3];
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
-        w[j] = sc.limb(kVjpU + 4 * j + g);
-        const int64_t x = whole(w[j]);
+        const int64_t x = shr(sc.get(kVjpU + 4 * j + g), kap - (eu[j] + t[j]));
+        w[j] = limb(x);
         wn[j] = limb(shl(x, n));
         const int64_t y = shr(mul8(tl, wn[j]), k);
         Tc[j] += y;
         v[j] = limb(y);
         V[j] += x;
       }
+      mac(q[0], v[0], w[0]);
+      mac(q[1], v[1], w[1]);
+      mac(q[2], v[2], w[2]);
+      mac(q[3], v[0], w[1]);
+      mac(q[4], v[0], w[2]);
+      mac(q[5], v[1], w[2]);
       if constexpr (INT) {
         // alpha u_g-bar = tau (alpha Tb + 2 N) + alpha^2 sc W, N = alpha^2 Qh W,
         // alpha^2 sc = (alpha^2 k2 / |u_g|) (-tau^2) (staub + W . (alpha Tb + N))
@@ -342,23 +345,23 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
         int64_t ym = scalar_fixed(yd, ey);
         if (yd == 0.0) ym = 0;  // at rest
         const Limb ty = limb(mul8(limb(mul8(tl, limb(tm * 2))), limb(ym * 2)));
-        const Limb s2 = limb(-mul8(ty, limb(shl(tb, nb))));
-        const int es = 2 * et + ey + eb - nb + 6 + kap - n;
+        const int64_t sw = -mul8(ty, limb(shl(tb, nb)));
+        const int ns = norm_shift(mag(sw)) - 1;
+        const Limb s2 = limb(shl(sw, ns));
+        const int es = 2 * et + ey + eb - nb + 6 - ns;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-          const int64_t x = mul8(tl, limb(N[i])), y = mul8(s2, wn[i]);
-          const int nx = norm_shift(mag(x)), ny = norm_shift(mag(y));
-          const int ex = et + eY + t[i] - nx, ey = es - t[i] - ny, e = imax(ex, ey) + 1;
-          sc.put(kVjpX + 3 * g + i, shr(shl(x, nx), e - ex) + shr(shl(y, ny), e - ey));
+          // the last term takes W as it is, not the aligned W~, which has lost a
+          // bit per factor 2 of the cell's flatness
+          const int64_t u = sc.get(kVjpU + 4 * i + g);
+          const int nu = norm_shift(mag(u));
+          const int64_t x = mul8(tl, limb(N[i])), y = mul8(s2, limb(shl(u, nu)));
+          const int nx = norm_shift(mag(x));
+          const int ex = et + eY + t[i] - nx, ey = es + eu[i] - nu, e = imax(ex, ey) + 1;
+          sc.put(kVjpX + 3 * g + i, shr(shl(x, nx), e - ex) + shr(y, e - ey));
           sc.put_word(kVjpXg + 3 * g + i, e);
         }
       }
-      mac(q[0], v[0], w[0]);
-      mac(q[1], v[1], w[1]);
-      mac(q[2], v[2], w[2]);
-      mac(q[3], v[0], w[1]);
-      mac(q[4], v[0], w[2]);
-      mac(q[5], v[1], w[2]);
     }
     Limb a1l = P.a1.m;
     int ea1 = P.a1.e + einv;
@@ -371,14 +374,15 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
       }
     }
     gauss_matrices(q, Tc, theta, kap, inv, einv, mul8(inv, a1l), ea1, t, tmax, P, Qp, eP, sT, eT);
-    // W~_a back to u_a = W_a - QB sum_b W_b (the sum is S sqrt 5)
+    // from W~_a to u_a = W_a - QB sum_b W_b (the sum is S sqrt 5)
 #pragma unroll
     for (int j = 0; j < 3; ++j) V[j] = qb_sum(V[j]);
 #pragma unroll 1
     for (int a = 0; a < 4; ++a)
 #pragma unroll
       for (int j = 0; j < 3; ++j)
-        sc.put(kVjpU + 4 * j + a, limb(whole(sc.limb(kVjpU + 4 * j + a)) - V[j]));
+        sc.put(kVjpU + 4 * j + a,
+               limb(shr(sc.get(kVjpU + 4 * j + a), kap - (eu[j] + t[j])) - V[j]));
     if constexpr (INT) {
       // (QA - QB) u_a-bar + QB sum_g u_g-bar, QB = alpha beta
 #pragma unroll 1

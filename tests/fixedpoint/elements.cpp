@@ -140,6 +140,94 @@ static void wall_cell() {
   say("wall_cell", 0, 0, s.worst(), 1e-12);
 }
 
+// Flat cells: component i of the velocity of size scale^i; scale 0: normal
+// deviates, some Gauss points of which are nearly at rest. In place, against the
+// element in long double, where the double-precision routine's own error (10 %
+// for the spread of a finite sample) is the limit, as in check.cpp; rotated,
+// where the rounded geometry is common to both, against that routine: two
+// results whose errors are a few 1e-16 each.
+static Element flat_cell(double flat, double scale, bool rotated) {
+  Element q = make(0, 0);
+  double R[3][3];
+  const double a = rotated ? uni(0, 6.3) : 0, b = rotated ? uni(0, 6.3) : 0;
+  const double A[3][3] = {{std::cos(a), -std::sin(a), 0}, {std::sin(a), std::cos(a), 0}, {0, 0, 1}};
+  const double B[3][3] = {{std::cos(b), 0, std::sin(b)}, {0, 1, 0}, {-std::sin(b), 0, std::cos(b)}};
+  for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j) R[i][j] = A[i][0] * B[0][j] + A[i][1] * B[1][j] + A[i][2] * B[2][j];
+  for (int n = 0; n < 4; ++n) {
+    const double x[3] = {q.X[n][0], q.X[n][1], q.X[n][2] / flat};
+    for (int i = 0; i < 3; ++i) {
+      q.X[n][i] = R[i][0] * x[0] + R[i][1] * x[1] + R[i][2] * x[2];
+      q.u[n][i] = scale > 0 ? (1 + uni(-0.9, 0.9)) * std::pow(scale, i) : normal();
+    }
+  }
+  element_geometry<double, double>(q.X, q.c, q.inv, q.rh);
+  q.P.mu = 1e-4;  // tau from the velocity rather than from the viscosity
+  return q;
+}
+template <int FLAGS>
+static void exact_element(const Element& q, ld rhs[4][4], ld vjp[4][4]) {
+  typedef std::complex<ld> cld;
+  const ld step = 1e-30L;
+  for (int b = -1; b < 4; ++b)
+    for (int k = 0; k < (b < 0 ? 1 : 4); ++k) {
+      cld u[4][3], p[4], F[4][4];
+      for (int a = 0; a < 4; ++a) {
+        for (int i = 0; i < 3; ++i) u[a][i] = cld(q.u[a][i], a == b && i == k ? step : 0);
+        p[a] = cld(q.p[a], a == b && k == 3 ? step : 0);
+      }
+      reference<FLAGS, cld>(q.X, u, p, q.P, F);
+      if (b >= 0) vjp[b][k] = 0;
+      for (int a = 0; a < 4; ++a)
+        for (int i = 0; i < 4; ++i) {
+          if (b < 0) rhs[a][i] = F[a][i].real();
+          else vjp[b][k] += q.w[a][i] * (F[a][i].imag() / step);
+        }
+    }
+}
+// Errors of a routine against long double, norm-wise per component.
+struct Error {
+  double d[8] = {}, n[8] = {};
+  void add(const Results& x, const ld rhs[4][4], const ld vjp[4][4]) {
+    for (int a = 0; a < 4; ++a)
+      for (int k = 0; k < 4; ++k) {
+        d[k] += std::pow((double)(x.rhs[a][k] - rhs[a][k]), 2);
+        n[k] += std::pow((double)rhs[a][k], 2);
+        d[4 + k] += std::pow((double)(x.vjp[a][k] - vjp[a][k]), 2);
+        n[4 + k] += std::pow((double)vjp[a][k], 2);
+      }
+  }
+  double of(int k) const { return n[k] > 0 ? std::sqrt(d[k] / n[k]) : 0.0; }
+};
+template <int FLAGS>
+static void flat_cells(int n) {
+  for (const double flat : {1.0, 20.0, 100.0, 1e3, 1e4})
+    for (const double scale : {1.0, 1e-6, 0.0}) {
+      if (scale < 1 && (FLAGS & kSkew)) continue;  // the sweep is in double precision there
+      const int id = (int)flat * 10 + (scale == 0 ? 2 : scale < 1);
+      Error mine, ref;
+      Sum turned;
+      for (int it = 0; it < n; ++it) {
+        Element q = flat_cell(flat, scale, false);
+        Results x, y;
+        ld rhs[4][4], vjp[4][4];
+        by_double<FLAGS>(q, y);
+        if (!by_fixed<FLAGS>(q, x)) say("flat_cell_left", FLAGS, id, 1, 0);
+        exact_element<FLAGS>(q, rhs, vjp);
+        mine.add(x, rhs, vjp);
+        ref.add(y, rhs, vjp);
+        if (scale < 1) continue;
+        q = flat_cell(flat, scale, true);
+        by_double<FLAGS>(q, y);
+        if (!by_fixed<FLAGS>(q, x)) say("flat_cell_left", FLAGS, id, 1, 0);
+        turned.add(x, y);
+      }
+      for (int k = 0; k < 8; ++k)
+        say(k < 4 ? "flat_cell_rhs" : "flat_cell_vjp", FLAGS, 10 * id + k, mine.of(k), 1.1 * ref.of(k));
+      if (scale == 1) say("flat_cell_rotated", FLAGS, id, turned.worst(), 2e-15);
+    }
+}
+
 template <int FLAGS>
 static void all(int n) {
   expectations<FLAGS>(n / 10);
@@ -148,6 +236,10 @@ static void all(int n) {
 
 int main() {
   wall_cell();
+  flat_cells<0>(2000);
+  flat_cells<kSkew>(1000);
+  flat_cells<kTauElem>(1000);
+  flat_cells<kSkew | kTauElem>(1000);
   all<0>(100000);
   all<1>(20000);
   all<2>(20000);
