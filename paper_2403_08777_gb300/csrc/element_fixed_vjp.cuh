@@ -65,6 +65,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
 
   // ---- nodal values of u, v, w, p and the cotangent (real U 2^(e_i - 59)):
   // gradient rows (real R 2^(eg_i + t_j - 61)), W of the velocities ----
+  uint32_t least = ~0u;
 #pragma unroll 1
   for (int i = 0; i < 8; ++i) {
     const int at = i < 3 ? kVjpU + 4 * i : i == 3 ? kVjpP : kVjpW + 4 * (i - 4);
@@ -87,6 +88,7 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
 #pragma unroll
     for (int j = 0; j < 3; ++j) g[j] = dot3x<2>(Dl[0], C[0][j], Dl[1], C[1][j], Dl[2], C[2][j]);
     const int n = norm_shift(mag(g[0]) | mag(g[1]) | mag(g[2]));
+    least = umin(least, umin(umin(mag(g[0]), mag(g[1])), mag(g[2])));
 #pragma unroll
     for (int j = 0; j < 3; ++j) sc.put(kVjpR + 3 * i + j, shl(g[j], n));
     sc.put_word(kVjpEg + i, (sh < 0 ? kZeroExp : E - 1021 - sh) + 2 - n);
@@ -102,7 +104,6 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
       for (int a = 0; a < 4; ++a) sc.put(at + a, U[a] + s);
     }
   }
-  if (!ok) return false;
   int t[3], eu[3], eG[3], eO[3], ew[3];
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
@@ -114,6 +115,8 @@ __device__ __forceinline__ bool element_vjp_fixed(const Scratch<THREADS>& sc, do
   }
   const int egp = sc.word(kVjpEg + 3), ecw = sc.word(kVjpEg + 7);
   const int tmax = imax(t[0], imax(t[1], t[2]));
+  ok = aligned_rows(sc, kVjpR, 8, 4, eu, t, tmax, least) && ok;
+  if (!ok) return false;
   const int eum = imax(eu[0], imax(eu[1], eu[2]));
   const int kap = imax(eu[0] + t[0], imax(eu[1] + t[1], eu[2] + t[2]));
   auto row = [&](int i, int j) { return sc.get(kVjpR + 3 * i + j); };

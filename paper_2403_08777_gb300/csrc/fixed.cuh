@@ -47,6 +47,9 @@ __device__ __forceinline__ uint32_t lo_word(double x) { return (uint32_t)__doubl
 __device__ __forceinline__ double make_double(uint64_t b) { return __longlong_as_double((long long)b); }
 __device__ __forceinline__ int clz32(uint32_t x) { return __clz((int)x); }
 __device__ __forceinline__ int imax(int a, int b) { return max(a, b); }
+__device__ __forceinline__ uint32_t umin(uint32_t a, uint32_t b) { return min(a, b); }
+// Whether x holds in any thread of the warp that is here: a branch that the warp takes together.
+__device__ __forceinline__ bool any_lane(bool x) { return __any_sync(__activemask(), x) != 0; }
 // a b + c, one instruction.
 __device__ __forceinline__ int64_t mad_wide(int32_t a, int32_t b, int64_t c) {
   int64_t d;
@@ -76,6 +79,8 @@ inline uint32_t lo_word(double x) { return (uint32_t)bits_of(x); }
 inline double make_double(uint64_t b) { double x; std::memcpy(&x, &b, 8); return x; }
 inline int clz32(uint32_t x) { return x ? __builtin_clz(x) : 32; }
 inline int imax(int a, int b) { return a > b ? a : b; }
+inline uint32_t umin(uint32_t a, uint32_t b) { return a < b ? a : b; }
+inline bool any_lane(bool x) { return x; }
 inline int64_t mad_wide(int32_t a, int32_t b, int64_t c) {
   int64_t d;
   const bool over = __builtin_add_overflow((int64_t)a * b, c, &d);
@@ -108,6 +113,9 @@ __device__ __forceinline__ int64_t shr_round(int64_t x, int k) { return (shr(x *
 // Exponents of groups that hold only zeros: far below every other one, so
 // that such a group never decides an alignment.
 constexpr int kZeroExp = -4000;
+
+// Exponent (E - 1022 of group_exp) of a group of zeros.
+constexpr int kRestExp = 128 - 1022;
 
 __device__ __forceinline__ int32_t hi_abs(double x) { return hi_word(x) & 0x7fffffff; }
 

@@ -228,6 +228,77 @@ static void flat_cells(int n) {
     }
 }
 
+// Fields that do not vary along an axis, in cells flat or long along it: 0 nothing
+// varies, the velocity in the plane only; 1 with a constant velocity across; 2 with
+// one that varies in the plane; 3 the cotangent alone does not vary; 4 a channel,
+// the velocity u(z) and the pressure p(x). Where the double-precision sums are
+// exact, a sum may lose 6 of the 59 bits that its terms have: 2^-53 for each of
+// the at most 32 products of a row. Where the double-precision routine has a larger
+// error, 4 times that, for the one element that decides a sum over few.
+static Element layered(int kind, int axis, double stretch) {
+  Element q;
+  const Element any = make(0, 0);
+  static const int perm[6][3] = {{0, 1, 2}, {1, 2, 0}, {2, 0, 1}, {0, 2, 1}, {2, 1, 0}, {1, 0, 2}};
+  const int t = (int)(rng() % 6);
+  int l[4][3] = {};
+  for (int s = 0; s < 3; ++s) {
+    for (int d = 0; d < 3; ++d) l[s + 1][d] = l[s][d];
+    l[s + 1][perm[t][s]] += 1;
+  }
+  if (t >= 3)
+    for (int d = 0; d < 3; ++d) std::swap(l[1][d], l[2][d]);
+  double field[8][8], off[8][3], at[3];
+  for (auto& r : field)
+    for (double& x : r) x = normal();
+  for (auto& r : off)
+    for (double& x : r) x = 0.12 * uni(-1, 1);
+  for (double& x : at) x = std::floor(uni(0, 64));
+  const int across = 1 << axis;
+  for (int a = 0; a < 4; ++a) {
+    const int id = l[a][0] | l[a][1] << 1 | l[a][2] << 2, in = id & ~across;
+    for (int d = 0; d < 3; ++d)
+      q.X[a][d] = (l[a][d] + at[d] + (d == axis ? 0.0 : off[in][d])) / 64 * (d == axis ? stretch : 1);
+    for (int k = 0; k < 8; ++k) {
+      const bool varies = k > 3 ? kind == 4 : kind == 3;
+      double x = field[k][varies ? id : in];
+      if (kind == 4 && k < 4) x = field[k][id & (k == 0 ? across : 1 << (axis + 1) % 3)];
+      if (k == axis && kind < 2) x = kind;
+      if (kind == 4 && k < 3) x = k == 0 ? 0.5 + std::fabs(x) : 0.0;
+      if (k < 3) q.u[a][k] = x;
+      else if (k == 3) q.p[a] = x;
+      else q.w[a][k - 4] = x;
+    }
+  }
+  element_geometry<double, double>(q.X, q.c, q.inv, q.rh);
+  q.P = any.P;
+  q.P.mu = rng() & 1 ? 1e-2 : 1e-4;
+  return q;
+}
+template <int FLAGS>
+static void layers(int n) {
+  for (int kind = 0; kind < 5; ++kind)
+    for (int axis = 0; axis < 3; ++axis)
+      for (const double stretch : {1.0, 0.1, 1e-2, 1e-3, 1e-4, 1e2, 1e4}) {
+        Error mine, ref;
+        g_violations = 0;
+        for (int it = 0; it < n; ++it) {
+          const Element q = layered(kind, axis, stretch);
+          Results x, y;
+          ld rhs[4][4], vjp[4][4];
+          by_double<FLAGS>(q, y);
+          if (!by_fixed<FLAGS>(q, x)) x = y;  // as the kernels do
+          exact_element<FLAGS>(q, rhs, vjp);
+          mine.add(x, rhs, vjp);
+          ref.add(y, rhs, vjp);
+        }
+        const int id = (kind * 3 + axis) * 100 + (int)std::lround(10 * std::log10(stretch));
+        for (int k = 0; k < 8; ++k)
+          say(k < 4 ? "layered_rhs" : "layered_vjp", FLAGS, id * 10 + k, mine.of(k),
+              std::max(32 * 0x1p-53, 4 * ref.of(k)));
+        say("layered_expect", FLAGS, id, (double)g_violations, 0);
+      }
+}
+
 template <int FLAGS>
 static void all(int n) {
   expectations<FLAGS>(n / 10);
@@ -240,6 +311,10 @@ int main() {
   flat_cells<kSkew>(1000);
   flat_cells<kTauElem>(1000);
   flat_cells<kSkew | kTauElem>(1000);
+  layers<0>(60);
+  layers<kSkew>(30);
+  layers<kTauElem>(30);
+  layers<kSkew | kTauElem>(30);
   all<0>(100000);
   all<1>(20000);
   all<2>(20000);

@@ -15,7 +15,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 @pytest.mark.skipif(shutil.which("g++") is None, reason="needs g++")
 def test_fixed_point_elements(tmp_path):
     exe = str(tmp_path / "elements")
-    subprocess.check_call(["g++", "-std=c++17", "-O2", "-Wno-unused-function",
+    subprocess.check_call(["g++", "-std=c++17", "-O2", "-ffp-contract=off", "-Wno-unused-function",
                            "-I" + os.path.join(HERE, "flopcount"), "-o", exe,
                            os.path.join(HERE, "fixedpoint", "elements.cpp")])
     out = subprocess.check_output([exe], text=True)
