@@ -87,9 +87,25 @@ FP64_LANES_PER_SM = 2
 # Warp instructions per 32 tets (smsp__inst_executed.sum of the same captures):
 # the FP64 kernels do most of the element in block fixed-point arithmetic on the
 # integer pipe, so their roof is the issue rate of the four schedulers of an SM,
-# not the FP64 pipe, which they pass (frac_fp64_pipe above 1).
+# not the FP64 pipe, which they pass (frac_fp64_pipe above 1). Of the default
+# formulation; None once a kernel has changed since its counters were taken.
 WARP_INSTR_PER_32_TETS = {"fwd_fp64": 4827, "vjp_fp64": 9699}
 WARP_INSTR_PER_SM_PER_CLOCK = 4
+
+
+def issue_roofline(key, ms, n_elems, n_sm, clk_mhz, default):
+    """An FP64 kernel's instructions against the issue rate; achieved and frac
+    None where they have not been counted: another formulation (not `default`),
+    or a kernel that has changed since."""
+    peak = WARP_INSTR_PER_SM_PER_CLOCK * n_sm * clk_mhz * 1e6 / 1e9
+    per = WARP_INSTR_PER_32_TETS.get(key) if default else None
+    ach = per * n_elems / 32 / (ms * 1e-3) / 1e9 if per else None
+    return {"bound": "alu", "kernel": key, "achieved": ach, "peak": peak,
+            "unit": "G warp instructions/s", "frac": ach / peak if per else None,
+            "peak_source": f"issue rate: {WARP_INSTR_PER_SM_PER_CLOCK} warp instructions per "
+                           f"SM and clock x {n_sm} SMs x {clk_mhz:.0f} MHz sampled during "
+                           f"the timed region",
+            "warp_instr_per_32_tets": per}
 
 
 def parse():
@@ -643,22 +659,14 @@ def run_ours(args):
             forms["partitioned_one_gpu"] = {"error": repr(exc)}
 
     # the FP64 kernels against the issue rate
-    issue_peak = WARP_INSTR_PER_SM_PER_CLOCK * n_sm * clk_mhz * 1e6 / 1e9
-
-    def issue_roofline(key, ms):
-        ach = WARP_INSTR_PER_32_TETS[key] * w.n_elems / 32 / (ms * 1e-3) / 1e9
-        return {"bound": "alu", "kernel": key, "achieved": ach, "peak": issue_peak,
-                "unit": "G warp instructions/s", "frac": ach / issue_peak,
-                "peak_source": f"issue rate: {WARP_INSTR_PER_SM_PER_CLOCK} warp instructions per "
-                               f"SM and clock x {n_sm} SMs x {clk_mhz:.0f} MHz sampled during "
-                               f"the timed region",
-                "warp_instr_per_32_tets": WARP_INSTR_PER_32_TETS[key],
+    def fp64_roofline(key, ms):
+        return {**issue_roofline(key, ms, w.n_elems, n_sm, clk_mhz, default=w.c_vreman == 0),
                 "tflops_algorithmic": forms[key]["tflops"],
                 "frac_fp64_pipe": forms[key]["frac_fp64_pipe"], "launch_ms": ms}
 
     dom = "vjp_fp64" if vjp_med >= fwd_med else "fwd_fp64"
     dom_ms = vjp_med if dom == "vjp_fp64" else fwd_med
-    roofline = issue_roofline(dom, dom_ms)
+    roofline = fp64_roofline(dom, dom_ms)
     roofline["traffic"] = (DRAM_BYTES_PER_TET[dom] * w.n_elems
                            if DRAM_BYTES_PER_TET.get(dom) is not None else None)
     roofline["flops_per_tet"] = flops["vjp" if dom == "vjp_fp64" else "fwd"]
@@ -681,7 +689,7 @@ def run_ours(args):
             "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": bench_config(w, world),
             "roofline": roofline,
-            "roofline_fwd": {**issue_roofline("fwd_fp64", fwd_med), "flops_per_tet": flops["fwd"],
+            "roofline_fwd": {**fp64_roofline("fwd_fp64", fwd_med), "flops_per_tet": flops["fwd"],
                              "flops_per_tet_method": mflops["fwd"],
                              "tflops_method": mflops["fwd"] * w.n_elems / (fwd_med * 1e-3) / 1e12},
             "roofline_mixed": roofline_mixed,
