@@ -89,7 +89,7 @@ FP64_LANES_PER_SM = 2
 # integer pipe, so their roof is the issue rate of the four schedulers of an SM,
 # not the FP64 pipe, which they pass (frac_fp64_pipe above 1). Of the default
 # formulation; None once a kernel has changed since its counters were taken.
-WARP_INSTR_PER_32_TETS = {"fwd_fp64": 4827, "vjp_fp64": 9699}
+WARP_INSTR_PER_32_TETS = {"fwd_fp64": 4850, "vjp_fp64": 9808}
 WARP_INSTR_PER_SM_PER_CLOCK = 4
 
 

@@ -216,12 +216,12 @@ nsrhs_status nsrhs_assemble_vjp(const nsrhs_mesh* m, const nsrhs_params* p, cons
                                 const void* cot, double* grad, void* stream);
 
 /*
- * Both of the above at the same state in one pass: rhs = assembled RHS of up
- * and grad = (d rhs / d up)^T cot, with one gather of up and cot per element
- * and the element's forward intermediates computed once (the adjoint's
- * recomputation of them is shared with the RHS); NSRHS_FP64 with atomics runs
- * the forward and the adjoint one after the other, which is faster. For callers that hold the
- * cotangent before the RHS is needed: residual and adjoint-residual sweeps
+ * Both of the above at the same state in one call: rhs = assembled RHS of up
+ * and grad = (d rhs / d up)^T cot. NSRHS_FP64 with atomics (AUTO) runs the
+ * forward and the adjoint one after the other; NSRHS_MIXED and the blocks make
+ * one pass, with one gather of up and cot per element and the element's forward
+ * intermediates computed once. For callers that hold the cotangent before the
+ * RHS is needed: residual and adjoint-residual sweeps
  * of steady adjoint solvers, one-shot optimisation, Newton-Krylov with a
  * transposed product. Types and layouts as nsrhs_assemble / _vjp; rhs and
  * grad must be distinct and are overwritten. Scatter AUTO (atomics for

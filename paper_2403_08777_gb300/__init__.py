@@ -177,8 +177,9 @@ class Mesh:
 
     def assemble_rhs_vjp(self, up: torch.Tensor, cot: torch.Tensor,
                          params: Params | None = None, *, out=None, **kw):
-        """(rhs, (d rhs / d up)^T cot) at the same state in one pass; both
-        [4, N] float64. out: optional pair of [4, N] float64 tensors."""
+        """(rhs, (d rhs / d up)^T cot) at the same state in one call (one pass
+        over the elements in mixed precision and with blocks; FP64 with atomics
+        the forward and then the adjoint); both [4, N] float64. out: optional pair of [4, N] float64 tensors."""
         p = self._params(params, kw)
         dt = torch.float32 if p.precision == "mixed" else torch.float64
         _require(up, "up", dt, (4, self.n_nodes), self.device)

@@ -22,8 +22,10 @@
 // loops over components, Gauss points and rows are therefore kept rolled,
 // their per-thread arrays in shared memory.
 //
-// Elements whose data are outside 2^-100 .. 2^100 (or not finite) are left to
-// the FP64 routines: the functions return false before writing anything.
+// Elements whose data are outside 2^-100 .. 2^100 (or not finite), and those
+// with a gradient that vanishes on the axis that decides an alignment
+// (aligned_rows), are left to the FP64 routines: the functions return false
+// before writing anything.
 #pragma once
 
 #include "element.cuh"

@@ -8,10 +8,11 @@
 // exactly the form of the forward's momentum and continuity rows.
 // FP64 pipe: tau at the Gauss points, and the reverse sweep there with the
 // eddy viscosity, the skew-symmetric term or the per-element tau. Without
-// these the sweep has integer operands only, and an FP64 instruction costs
-// about five issue slots, so it runs on the integer pipe as well: 256^3 52.2
-// -> 46.3 ms. Its terms mix the scaling of gradients and of velocities; each
-// is normalised by itself, per Gauss point and component, before two meet.
+// these the sweep has integer operands only, and an FP64 instruction takes its
+// pipe 64 clocks, so it runs on the integer pipe as well: 256^3 52.2 -> 46.3
+// ms (48.3 with the tau term's velocity at full width). Its terms mix the
+// scaling of gradients and of velocities; each is normalised by itself, per
+// Gauss point and component, before two meet.
 #pragma once
 
 #include "element_fixed.cuh"

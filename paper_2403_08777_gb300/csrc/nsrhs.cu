@@ -602,10 +602,10 @@ constexpr int kFixedThreads = 32;
 // address receives at most one atomic in the launch and the colour order
 // fixes the summation order (bitwise reproducible).
 //
-// Bound by instruction issue (ALU pipe 60 % busy, 4650 instructions a warp at
-// 0.55 per clock and sub-partition), where the FP64 form kept the FP64 pipe
+// Bound by instruction issue (ALU pipe 62 % busy, 4850 instructions a warp at
+// 0.56 per clock and sub-partition), where the FP64 form kept the FP64 pipe
 // 90 % busy with 344 FP64 instructions (64 clocks of a sub-partition each):
-// 256^3 61.3 -> 20.5 ms.
+// 256^3 61.3 -> 20.4 ms.
 //
 // plain: every element on the FP64 pipe (parameters outside the fixed-point
 // range). chain: (u, p) comes from the launch before this one.
@@ -783,7 +783,7 @@ struct NodalVelocity {
 // with 18 KB of scratch a warp, where slots are laid over one another and
 // tau W~ is formed twice rather than kept; 10 with 22 KB took 128^3 7.67 ms,
 // 12 took 7.08 ms. The FP64 form kept the FP64 pipe 90 % busy with 648
-// instructions: 256^3 114.4 -> 46.3 ms.
+// instructions: 256^3 114.4 -> 48.3 ms (9808 instructions a warp).
 template <int FLAGS, class GS>
 __global__ void __launch_bounds__(kFixedThreads, 12)
     vjp_fp64_kernel(int64_t N, int64_t E, int64_t e0, int64_t e1,
@@ -886,7 +886,7 @@ __global__ void __launch_bounds__(kThreads)
 // (element_rhs_vjp): one gather of (u, p) and the cotangent, one geometry
 // read, the forward intermediates computed once; float arithmetic, double
 // accumulation by integer widening. (The FP64 form runs its forward and its
-// adjoint kernel one after the other: fixed-point forward and adjoint, 20.5 + 46.3
+// adjoint kernel one after the other: fixed-point forward and adjoint, 20.4 + 48.3
 // ms at 256^3, against 141 ms for one FP64 pass.)
 template <int FLAGS>
 __global__ void __launch_bounds__(kThreads)
@@ -1534,7 +1534,8 @@ nsrhs_status assemble(const nsrhs_mesh* m, const nsrhs_params* p, const void* up
     return cuda_status(err);
   }
   if (p->scatter == NSRHS_SCATTER_BLOCK_COLOUR) {
-    // one launch per block colour, in colour order
+    // one launch per block colour, in colour order; none is empty (a block takes the
+    // smallest colour absent at its nodes, so that colour's predecessor is in use)
     const int64_t nb = m->n_blocks;
     for (size_t k = 0; k + 1 < m->bcol_off.size() && err == cudaSuccess; ++k) {
       const int64_t i0 = m->bcol_off[k], i1 = m->bcol_off[k + 1];
